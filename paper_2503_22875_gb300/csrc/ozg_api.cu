@@ -56,15 +56,30 @@ int emu_gemm(ozg_ctx* c, bool cplx, char ta, char tb, int64_t m, int64_t n, int6
     const int64_t tiles = ((prA + BM - 1) / BM) * ((prB + BN - 1) / BN);
     return (int)(tiles < c->num_sms ? tiles : c->num_sms);
   };  // depends on the tile width (bit 0) only
-  const int grid = grid_of(0) > grid_of(1) ? grid_of(0) : grid_of(1);  // R scratch for either width
+  const int grid_kd = (int)std::min<int64_t>(2 * ozg::kd_tiles(prA, prB), c->num_sms / 2 * 2);
+  // difference planes up to kd slices (0: none): a fixed count's own, or every learned count that
+  // the difference-plane kernel takes
+  int kd = Gdbg ? 0 : choose_kd(c, cplx, prA, prB, k, autos ? std::min(c->sel_s_hi, ozg::kKdMax) : s, s);
+  int nplanes;
   Carve cv;
-  size_t oDA = cv.take((size_t)s * prA * Kp * 2), oDB = cv.take((size_t)s * prB * Kp * 2);
-  size_t oE = cv.take(4 * (size_t)m), oF = cv.take(4 * (size_t)n);
-  size_t oMA = cv.take(8 * (size_t)m), oMB = cv.take(8 * (size_t)n);
-  size_t oR = cv.take((size_t)grid * BM * 256 * 16);  // 16 bytes per output (128-bit Horner sum)
-  size_t oCold = cv.take((size_t)(nsamp > 0 ? nsamp : 1) * 16);
-  size_t oHist = cv.take(2 * 10 * 8), oSd = cv.take(4 * sizeof(int)), oErr2 = cv.take(sizeof(double));
-  size_t oSaved = cv.take((autos && !beta_zero0) ? (size_t)m * n * (cplx ? 16 : 8) : 8);
+  size_t oDA, oDB, oE, oF, oMA, oMB, oR, oCold, oHist, oSd, oErr2, oSaved;
+  auto layout = [&]() {
+    nplanes = ozg::kd_planes(s, kd);
+    const int grid = std::max({grid_of(0), grid_of(1), kd ? grid_kd : 0});  // R scratch for every kernel
+    cv = Carve();
+    oDA = cv.take((size_t)nplanes * prA * Kp * 2), oDB = cv.take((size_t)nplanes * prB * Kp * 2);
+    oE = cv.take(4 * (size_t)m), oF = cv.take(4 * (size_t)n);
+    oMA = cv.take(8 * (size_t)m), oMB = cv.take(8 * (size_t)n);
+    oR = cv.take((size_t)grid * BM * 256 * 16);  // 16 bytes per output (128-bit Horner sum)
+    oCold = cv.take((size_t)(nsamp > 0 ? nsamp : 1) * 16);
+    oHist = cv.take(2 * 10 * 8), oSd = cv.take(4 * sizeof(int)), oErr2 = cv.take(sizeof(double));
+    oSaved = cv.take((autos && !beta_zero0) ? (size_t)m * n * (cplx ? 16 : 8) : 8);
+  };
+  layout();
+  if (kd && !ws_available(c, cv.off)) {  // without the differences where the memory is not there
+    kd = 0;
+    layout();
+  }
   int rc = ensure_ws(c, cv.off);
   if (rc) return rc;
   cudaStream_t st = c->stream;
@@ -87,6 +102,8 @@ int emu_gemm(ozg_ctx* c, bool cplx, char ta, char tb, int64_t m, int64_t n, int6
   sa.maxbits = at<unsigned long long>(c, oMA);
   sa.exps = at<int32_t>(c, oE);
   sa.nonfinite = nonfinite;
+  sa.kd = kd;
+  sa.diff = 1;
   // learned count: row maxima -> features -> selection -> digits up to the selected count only
   int* s_dev = at<int>(c, oSd);  // [0] chosen s, [1] 1 unless the check forced a re-run
   if (autos) sa.plane_to = s_dev;
@@ -100,6 +117,7 @@ int emu_gemm(ozg_ctx* c, bool cplx, char ta, char tb, int64_t m, int64_t n, int6
   sb.D = at<__half>(c, oDB);
   sb.maxbits = at<unsigned long long>(c, oMB);
   sb.exps = at<int32_t>(c, oF);
+  sb.diff = -1;
   // learned count with rows that fit a fused statistics unit: row maxima and features in one read
   const bool fused = autos && ozg::stats_fused(sa) && ozg::stats_fused(sb);
   unsigned long long* hist = at<unsigned long long>(c, oHist);
@@ -137,11 +155,11 @@ int emu_gemm(ozg_ctx* c, bool cplx, char ta, char tb, int64_t m, int64_t n, int6
   }
 
   CUtensorMap tmA, tmB[2];
-  OZG_CUDA(ozg::make_digit_tmap(&tmA, sa.D, k, prA, Kp, s, BM));
-  OZG_CUDA(ozg::make_digit_tmap(&tmB[0], sb.D, k, prB, Kp, s, ozg::slice_gemm_tile_n_of(0)));
-  OZG_CUDA(ozg::make_digit_tmap(&tmB[1], sb.D, k, prB, Kp, s, ozg::slice_gemm_tile_n_of(1)));
+  OZG_CUDA(ozg::make_digit_tmap(&tmA, sa.D, k, prA, Kp, nplanes, BM, kd != 0));
+  OZG_CUDA(ozg::make_digit_tmap(&tmB[0], sb.D, k, prB, Kp, nplanes, ozg::slice_gemm_tile_n_of(0), kd != 0));
+  OZG_CUDA(ozg::make_digit_tmap(&tmB[1], sb.D, k, prB, Kp, nplanes, ozg::slice_gemm_tile_n_of(1), kd != 0));
   // tmB[v & 1] serves variant v
-  int variant = choose_variant(c, prA, prB, k, s);
+  int variant = kd ? ozg::kStackedVariant : choose_variant(c, prA, prB, k, s);
   ozg::GemmArgs ga;
   ga.rows = prA;
   ga.cols = prB;
@@ -168,7 +186,8 @@ int emu_gemm(ozg_ctx* c, bool cplx, char ta, char tb, int64_t m, int64_t n, int6
   ga.grid = grid_of(variant);
   ga.s_dev = autos ? s_dev : nullptr;
   ga.exact = c->exact;
-  if (c->autotune && c->force_variant < 0 && !Gdbg && ga.beta_zero && !autos) {
+  ga.kd = kd;
+  if (c->autotune && !kd && c->force_variant < 0 && !Gdbg && ga.beta_zero && !autos) {
     const uint64_t bucket = shape_bucket(prA, prB, k, s);
     if (c->tune.find(bucket) == c->tune.end()) {
       // time the 1-CTA variants (two widths x stage shape or deferred pushes, and the stacked
@@ -238,7 +257,13 @@ int emu_gemm(ozg_ctx* c, bool cplx, char ta, char tb, int64_t m, int64_t n, int6
   }
   {
     PhaseScope ps(c, OZG_PHASE_GEMM);
-    OZG_CUDA(ozg::launch_slice_gemm(tmA, tmB[ga.variant & 1], ga, st));
+    if (kd) {
+      ozg::GemmArgs gd = ga;
+      gd.grid = grid_kd;
+      OZG_CUDA(ozg::launch_slice_gemm_kd(tmA, tmB[1], gd, st));  // tmB[1]: boxes of 128 columns
+    }
+    // a learned count above kd runs on the digit planes alone
+    if (!kd || (autos && s > kd)) OZG_CUDA(ozg::launch_slice_gemm(tmA, tmB[ga.variant & 1], ga, st));
   }
   if (Gdbg) return OZG_OK;
 
@@ -278,6 +303,7 @@ int emu_gemm(ozg_ctx* c, bool cplx, char ta, char tb, int64_t m, int64_t n, int6
     ca.plane_from = cb.plane_from = s_dev;
     ca.plane_to = cb.plane_to = nullptr;
     ca.gate = cb.gate = s_dev + 1;
+    ca.diff = cb.diff = 0;  // the re-run reads digit planes only
     OZG_CUDA(ozg::launch_digits(ca, st));
     OZG_CUDA(ozg::launch_digits(cb, st));
     ozg::GemmArgs g2 = ga;

@@ -106,6 +106,9 @@ struct Carve {
 };
 
 int ensure_ws(ozg_ctx* c, size_t bytes);
+// whether ensure_ws would find the memory: the workspace is large enough, or enough is free (and
+// the stream is not being captured, where it cannot grow)
+bool ws_available(ozg_ctx* c, size_t bytes);
 int ensure_gws(ozg_ctx* c, size_t bytes);  // grouped workspace; bumps gws_epoch when it moves
 int ensure_z3ws(ozg_ctx* c, size_t bytes);  // 3M operands and products
 cudaEvent_t pool_get(ozg_ctx* c);
@@ -131,6 +134,9 @@ T* gat(ozg_ctx* c, size_t off) {
 // tile variant for one GEMM shape (bit 0: BN = 128, bit 1: deferred pushes): the autotuned
 // choice if known, else the heuristic (least padding; deferral for k >= 2048)
 int choose_variant(ozg_ctx* c, int64_t rows, int64_t cols, int64_t k, int s);
+// slice count up to which one GEMM's planes include differences and the difference-plane kernel
+// runs (0: not at all); s: the fixed count or the largest learned one, s_planes: digit planes
+int choose_kd(ozg_ctx* c, bool cplx, int64_t rows, int64_t cols, int64_t k, int s, int s_planes);
 // grouped calls (ozg_grouped.cu): with sync_reports == false the reports are filled in by
 // grouped_collect_reports once the work has finished
 int grouped_call(ozg_ctx* c, int64_t count, const ozg_gemm_desc* descs, const int* slices, ozg_report* reps,

@@ -735,9 +735,11 @@ __device__ __forceinline__ void stacked_body(const CUtensorMap* tmA0, const CUte
                   const bool hasA = i >= 1, hasB = last ? kbi + 1 < KB : true;
                   const bool mirror = hasB && e == 0;
                   mbar_arrive_expect_tx(&bar_full[e], (hasA ? SLOT : 0u) + (hasB ? SLOT : 0u) + (mirror ? SLOT : 0u));
-                  if (hasA) tma_load_3d(j.tmA, &bar_full[e], smem + A_OFF + e * SLOT, kb * BK, arow, i - 1);
+                  if (hasA) tma_load_3d(j.tmA, &bar_full[e], smem + A_OFF + e * SLOT, kb * BK, arow,
+                                        GROUPED ? i - 1 : kd_plane(i, j.kd));
                   if (hasB) {
-                    const int bk = (last ? kbn : kb) * BK, bz = last ? ga - 1 : ga - i - 1;
+                    const int bk = (last ? kbn : kb) * BK, t = last ? ga : ga - i;
+                    const int bz = GROUPED ? t - 1 : kd_plane(t, j.kd);
                     tma_load_3d(j.tmB, &bar_full[e], smem + B_OFF + e * SLOT, bk, brow, bz);
                     if (mirror) tma_load_3d(j.tmB, &bar_full[e], smem + B_OFF + NE * SLOT, bk, brow, bz);
                   }
@@ -1118,6 +1120,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     slice_gemm_stacked_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                               const GemmArgs P) {
   if (P.nonfinite != nullptr && *P.nonfinite) return;
+  if (P.kd != 0 && P.s_dev != nullptr && *P.s_dev <= P.kd) return;  // the difference-plane launch runs
   stacked_body<false>(&tmA, &tmB, &P, nullptr);
 }
 __global__ void __launch_bounds__(THREADS, 1) slice_gemm_grouped_stacked_kernel(const GroupArgs G) {
@@ -1191,11 +1194,11 @@ size_t slice_gemm_smem_bytes() { return Cfg<256, 1>::SMEM; }
 // promotion: the 8192^3 launch is 19.5 -> 18.9 ms).
 constexpr int64_t kWidePromotionMinK = 2049;
 cudaError_t make_digit_tmap(CUtensorMap* map, const __half* D, int64_t k, int64_t rows, int64_t Kp, int s,
-                            int box_rows) {
+                            int box_rows, bool forward) {
   EncodeTiledFn enc = get_encode_fn();
   if (!enc) return cudaErrorNotSupported;
   const CUtensorMapL2promotion promo =
-      k >= kWidePromotionMinK ? CU_TENSOR_MAP_L2_PROMOTION_L2_256B : CU_TENSOR_MAP_L2_PROMOTION_L2_128B;
+      forward || k >= kWidePromotionMinK ? CU_TENSOR_MAP_L2_PROMOTION_L2_256B : CU_TENSOR_MAP_L2_PROMOTION_L2_128B;
   cuuint64_t dims[3] = {(cuuint64_t)k, (cuuint64_t)rows, (cuuint64_t)s};
   cuuint64_t strides[2] = {(cuuint64_t)Kp * 2, (cuuint64_t)(rows * Kp * 2)};
   cuuint32_t box[3] = {(cuuint32_t)BK, (cuuint32_t)box_rows, 1};
@@ -1252,6 +1255,7 @@ cudaError_t launch_variant(int variant, const CUtensorMap* tmA, const CUtensorMa
 // Shared-memory opt-in for every kernel instance, once per process (outside any graph capture).
 cudaError_t prepare_kernels() {
   cudaError_t e;
+  if ((e = prepare_kd_kernels()) != cudaSuccess) return e;
   if ((e = cudaFuncSetAttribute(slice_gemm_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)Cfg<128, 2, true>::SMEM)) != cudaSuccess)
     return e;
@@ -1282,6 +1286,9 @@ cudaError_t prepare_kernels() {
 
 cudaError_t launch_slice_gemm(const CUtensorMap& tmA, const CUtensorMap& tmB, const GemmArgs& a, cudaStream_t st) {
   if (a.grid <= 0) return cudaSuccess;
+  // a plane set with differences is read by the stacked kernel only
+  if (a.kd != 0 && (a.variant != kStackedVariant || a.exact || a.Gdbg != nullptr || a.s > stacked_max_slices()))
+    return cudaErrorInvalidValue;
   // the stacked kernel has no exact 128-bit mode and no group-product export; both, and slice
   // counts above its limit, run on the 128-wide one-group kernel (same tiles, same bits)
   const int v = (a.variant == kStackedVariant && (a.exact || a.Gdbg != nullptr || a.s > stacked_max_slices()))

@@ -1,4 +1,4 @@
-// Device code shared by the slice-product kernels (ozg_gemm.cu): the pipeline
+// Device code shared by the slice-product kernels (ozg_gemm.cu, ozg_gemm_kd.cu): the pipeline
 // constants, the description of one output tile from either work source, and the epilogue's
 // window arithmetic and final rounding of C.
 #pragma once
@@ -51,7 +51,7 @@ struct Cfg {
 struct TileJob {
   const CUtensorMap* tmA;
   const CUtensorMap* tmB;
-  int tm, tn, KB, s, cplx, skip;
+  int tm, tn, KB, s, cplx, skip, kd;
   int klast;  // 64-wide sub-tiles holding valid k in the last stage (1 .. SUB)
   int64_t rows, cols, n;  // stacked product rows / cols, output columns (complex: n)
   const int32_t* e;
@@ -72,18 +72,19 @@ __device__ __forceinline__ void tile_coords(int t, int tiles_m, int tiles_n, int
   tn = r / gsz;
 }
 
-template <int BN_, int SUB_, bool GROUPED, bool PAIR = false>
+template <int BN_, int SUB_, bool GROUPED, bool PAIR = false, int TROWS = BM>
 __device__ __forceinline__ TileJob get_job(int t, const CUtensorMap* tmA, const CUtensorMap* tmB, const GemmArgs* P,
                                            const GroupArgs* G) {
   TileJob j;
   if (!GROUPED) {
-    const int tiles_m = (int)((P->rows + BM - 1) / BM), tiles_n = (int)((P->cols + BN_ - 1) / BN_);
+    const int tiles_m = (int)((P->rows + TROWS - 1) / TROWS), tiles_n = (int)((P->cols + BN_ - 1) / BN_);
     tile_coords(t, tiles_m, tiles_n, j.tm, j.tn);
     j.tmA = tmA;
     j.tmB = tmB;
     j.KB = (int)((P->k + Cfg<BN_, SUB_>::SK - 1) / Cfg<BN_, SUB_>::SK);
     j.klast = (int)((P->k - (int64_t)(j.KB - 1) * Cfg<BN_, SUB_>::SK + BK - 1) / BK);
     j.s = P->s_dev != nullptr ? *P->s_dev : P->s;
+    j.kd = P->kd;
     j.cplx = P->cplx;
     j.skip = 0;
     j.rows = P->rows;
@@ -112,6 +113,7 @@ __device__ __forceinline__ TileJob get_job(int t, const CUtensorMap* tmA, const 
     j.KB = (int)((c->k + Cfg<BN_, SUB_>::SK - 1) / Cfg<BN_, SUB_>::SK);
     j.klast = (int)((c->k - (int64_t)(j.KB - 1) * Cfg<BN_, SUB_>::SK + BK - 1) / BK);
     j.s = c->s;
+    j.kd = c->kd;
     j.cplx = c->cplx;
     j.skip = (c->nonfinite != nullptr && *c->nonfinite) ? 1 : 0;
     j.rows = c->rows;

@@ -1,5 +1,6 @@
 // Host-side helpers shared by the C ABI translation units: CUDA error capture, workspace
 // growth, per-phase event timing, and the tile-variant autotuner's cache.
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -58,6 +59,21 @@ static int grow_buffer(ozg_ctx* c, void** buf, size_t* cap, size_t bytes) {
   }
   *cap = want;
   return OZG_OK;
+}
+
+bool ws_available(ozg_ctx* c, size_t bytes) {
+  if (bytes <= c->ws_cap) return true;
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(c->stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
+    cudaGetLastError();
+    return false;  // no growing while the caller captures: keep to what was reserved
+  }
+  size_t free_b = 0, total_b = 0;
+  if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return bytes + bytes / 8 + ((size_t)64 << 20) <= free_b + c->ws_cap;
 }
 
 int ensure_ws(ozg_ctx* c, size_t bytes) { return grow_buffer(c, &c->ws, &c->ws_cap, bytes); }
@@ -155,6 +171,41 @@ int choose_variant(ozg_ctx* c, int64_t rows, int64_t cols, int64_t k, int s) {
   // 2048^3 and for 8192^3 at s = 10, by 6%)
   if (s <= stacked_max_slices() && !c->exact) return kStackedVariant;
   return heuristic_variant(rows, cols, k, s);
+}
+
+// Difference planes (ozg_gemm_kd.cu) or the stacked kernel: both times estimated in microseconds
+// from the tiles in whole waves and the costs measured per 64-wide k stage, per pass and per tile.
+//   stacked: 128 x 128 tiles on 152 CTAs, 0.275 per stage + 18 per tile (final rounding);
+//   difference planes: 256 x 256 tiles on 76 CTA pairs, 0.30 per stage, 2 s - 1 passes and a tile
+//   end of 36 (complex, whose window words stay in registers: 25); 3.3 per pass of a real tile
+//   (its sums enter windows in L2; those of the first window also the second's), 1 per complex
+//   one; and the split writes s^2 / 4 more planes (at 5.5 TB/s).
+// Measured against the stacked kernel on one GB300: real 2048 x 2048 at s = 7, k = 1024 / 2048 /
+// 4096: 0.95 / 1.09 / 1.21 of its speed, 8192^3 s = 7 1.41; complex 1024 x 1024 s = 7 k = 192 /
+// 1024: 1.10 / 1.36, 3616^3 1.51.
+int choose_kd(ozg_ctx* c, bool cplx, int64_t rows, int64_t cols, int64_t k, int s, int s_planes) {
+  if (c->force_variant >= 0 || c->exact || s_planes > stacked_max_slices()) return 0;
+  const int64_t KB = (k + 63) / 64;
+  // the exact sum must fit two windows (window_len of ozg_round.cuh), and R its int32
+  auto window = [&](int x) {
+    const unsigned long long gmax = (unsigned long long)x * (unsigned long long)(KB * 64) * 16129ull * (cplx ? 2 : 1);
+    return std::max((62 - (64 - __builtin_clzll(gmax))) / 7 + 1, 1);
+  };
+  auto fits = [&](int x) { return x <= 2 * window(x) && window(x) * k * (cplx ? 2 : 1) <= 130000; };
+  int kd = std::min(s, kKdMax);
+  while (kd > 0 && !fits(kd)) --kd;
+  if (kd < s && s == s_planes) return 0;  // a fixed count runs on one kernel
+  const int se = s == s_planes ? s : std::min(kd, 8);  // a learned count is 7 - 9 in practice
+  if (kd < se || kd == 0) return 0;
+  auto waves = [](int64_t tiles, int64_t units) { return (double)((tiles + units - 1) / units); };
+  const int products = se + se * se / 4, win = window(se), len0 = se <= win ? 0 : se - win;
+  int stages = 0;  // of the stacked kernel per 64-wide k sub-tile: groups in pairs from the last down
+  for (int g = se + 1; g >= 2; g -= 2) stages += g - 1;
+  const double stacked = waves(((rows + 127) / 128) * ((cols + 127) / 128), c->num_sms) * (0.275 * stages * (double)KB + 18.0);
+  const double diff = waves(kd_tiles(rows, cols), c->num_sms / 2) *
+                          (0.30 * products * (double)KB + (cplx ? 2 * se - 1 + 25.0 : 3.3 * (2 * se - 1 + len0) + 36.0)) +
+                      (double)(rows + cols) * (double)k * 2.0 * (products - se) / 5.5e6;
+  return diff < stacked ? kd : 0;
 }
 
 }  // namespace host

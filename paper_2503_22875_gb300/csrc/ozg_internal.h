@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <cstdint>
 
+#include "ozg_planes.h"
+
 namespace ozg {
 
 // ---------------------------------------------------------------------------------- split
@@ -36,6 +38,9 @@ struct SplitArgs {
   const int* plane_from = nullptr;
   const int* plane_to = nullptr;
   const int* gate = nullptr;
+  int kd = 0;    // plane layout: difference planes up to this slice count (0: digit planes only)
+  int diff = 0;  // +1: write the differences digit p - digit q, -1: digit q - digit p, 0: none; they
+                 // are written when t_hi <= kd
 };
 cudaError_t launch_split(const SplitArgs& a, cudaStream_t st);
 // the two passes of launch_split (row maxima; digits over the plane range of a)
@@ -69,14 +74,19 @@ struct GemmArgs {
   int defer = 0;                // 1: spread intermediate epilogue pushes over the next drains
   const int* s_dev = nullptr;   // if set, the slice count is read here (device-chosen); s = plane count
   int exact = 0;                // 1: exact 128-bit Horner sum and one rounding (s <= 13)
+  int kd = 0;                   // difference planes: the planes' layout is kd_plane's for this count
 };
+
+int64_t kd_tiles(int64_t rows, int64_t cols);  // 256 x 256 tiles, one CTA pair each
+cudaError_t prepare_kd_kernels();
+cudaError_t launch_slice_gemm_kd(const CUtensorMap& tmA, const CUtensorMap& tmB, const GemmArgs& a, cudaStream_t st);
 
 // Grouped (batched) GEMM: one persistent launch over the tiles of many independent problems.
 struct GroupCall {
   CUtensorMap tmA, tmB;         // digit planes of this call (64-byte aligned inside the struct)
   CUtensorMap tmBh;             // B planes with half-height boxes (the CTA-pair variant)
   int64_t rows = 0, cols = 0, m = 0, n = 0, k = 0;
-  int s = 0, cplx = 0, beta_zero = 1, pad = 0;
+  int s = 0, cplx = 0, beta_zero = 1, kd = 0;  // kd: as GemmArgs::kd
   const int32_t* e = nullptr;
   const int32_t* f = nullptr;
   double* C = nullptr;
@@ -115,7 +125,7 @@ cudaError_t prepare_kernels();
 int slice_gemm_tile_n_of(int variant);
 // Tensor maps over the digit planes: dims {k, rows, s}, box {64, 128 | 256, 1}, fp16, SW128.
 cudaError_t make_digit_tmap(CUtensorMap* map, const __half* D, int64_t k, int64_t rows, int64_t Kp, int s,
-                            int box_rows);
+                            int box_rows, bool forward = false);
 cudaError_t launch_slice_gemm(const CUtensorMap& tmA, const CUtensorMap& tmB, const GemmArgs& a, cudaStream_t st);
 int slice_gemm_tile_m();
 int slice_gemm_tile_n();

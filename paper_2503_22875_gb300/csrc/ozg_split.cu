@@ -20,6 +20,7 @@ struct PlaneRange {
   const int* from;
   const int* to;
   const int* gate;
+  int kd, diff;
   __device__ __forceinline__ bool resolve(int s, int& lo, int& hi) const {
     if (gate != nullptr && *gate) return false;
     lo = from != nullptr ? *from + 1 : 1;
@@ -27,6 +28,31 @@ struct PlaneRange {
     return lo <= hi;
   }
 };
+
+// The planes lo .. hi of eight consecutive elements b (bit patterns) of a row with exponent e.
+template <int KD>
+__device__ __forceinline__ void store_planes8(const uint64_t (&b)[8], int e, int lo, int hi, __half* out,
+                                              int64_t plane, const PlaneRange& pr) {
+  DigitSrc ds[8];
+  if (KD && pr.diff != 0 && hi <= pr.kd) {
+    if (hi <= 9) {
+#pragma unroll
+      for (int j = 0; j < 8; ++j) ds[j] = digit_src_first(b[j], e);
+      store_difference_planes<9>(ds, lo, hi, out, plane, pr.diff < 0);
+    } else {
+#pragma unroll
+      for (int j = 0; j < 8; ++j) ds[j] = digit_src(b[j], e);
+      store_difference_planes<kKdMax>(ds, lo, hi, out, plane, pr.diff < 0);
+    }
+    return;
+  }
+#pragma unroll
+  for (int j = 0; j < 8; ++j) ds[j] = digit_src(b[j], e);
+  if (KD)
+    store_digit_planes_kd<kMaxPlanes>(ds, lo, hi, out, plane, pr.kd);
+  else
+    store_digit_planes<kMaxPlanes>(ds, lo, hi, out, plane);
+}
 
 __device__ __forceinline__ void flag_nonfinite(uint64_t absbits, int* nonfinite) {
   if (absbits >= kInfBits) atomicExch(nonfinite, 1);
@@ -97,7 +123,7 @@ __global__ void rowmax_strided(const double* __restrict__ X, int64_t ld, int64_t
 
 // ---------------------------------------------------------------- digits, contiguous rows
 // thread per (row, group of 8 consecutive l); 16-byte stores per digit plane
-template <int CPLX>
+template <int CPLX, int KD>
 __global__ void digits_contig(const double* __restrict__ X, int64_t ld, int64_t rows, int64_t k, int conj, int s,
                               int64_t Kp, int64_t plane_rows, const unsigned long long* __restrict__ maxbits,
                               int32_t* __restrict__ exps, __half* __restrict__ D, PlaneRange pr) {
@@ -124,17 +150,14 @@ __global__ void digits_contig(const double* __restrict__ X, int64_t ld, int64_t 
   }
 #pragma unroll
   for (int part = 0; part < nparts; ++part) {
-    DigitSrc ds[8];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) ds[j] = digit_src(bits[part][j], e);
     int64_t orow = CPLX ? 2 * row + part : row;
-    store_digit_planes<kMaxPlanes>(ds, t_lo, t_hi, D + orow * Kp + l0, plane_rows * Kp);
+    store_planes8<KD>(bits[part], e, t_lo, t_hi, D + orow * Kp + l0, plane_rows * Kp, pr);
   }
 }
 
 // ---------------------------------------------------------------- digits, strided rows
 // block: 32 rows x 64 l tile staged (transposed) through shared memory
-template <int CPLX>
+template <int CPLX, int KD>
 __global__ void __launch_bounds__(256) digits_strided(const double* __restrict__ X, int64_t ld, int64_t rows,
                                                       int64_t k, int conj, int s, int64_t Kp, int64_t plane_rows,
                                                       const unsigned long long* __restrict__ maxbits,
@@ -174,11 +197,11 @@ __global__ void __launch_bounds__(256) digits_strided(const double* __restrict__
   if (l0 + lg == 0 && t_lo == 1) exps[row] = e;
 #pragma unroll
   for (int part = 0; part < W; ++part) {
-    DigitSrc ds[8];
+    uint64_t b[8];
 #pragma unroll
-    for (int j = 0; j < 8; ++j) ds[j] = digit_src(tile[lg + j][W * r + part], e);
+    for (int j = 0; j < 8; ++j) b[j] = tile[lg + j][W * r + part];
     int64_t orow = CPLX ? 2 * row + part : row;
-    store_digit_planes<kMaxPlanes>(ds, t_lo, t_hi, D + orow * Kp + l0 + lg, plane_rows * Kp);
+    store_planes8<KD>(b, e, t_lo, t_hi, D + orow * Kp + l0 + lg, plane_rows * Kp, pr);
   }
 }
 
@@ -216,28 +239,32 @@ cudaError_t launch_rowmax(const SplitArgs& a, cudaStream_t st) {
   return cudaGetLastError();
 }
 
+namespace {
+template <int CPLX, int KD>
+void digits_launch(const SplitArgs& a, cudaStream_t st) {
+  const PlaneRange pr{a.plane_from, a.plane_to, a.gate, a.kd, a.diff};
+  const int64_t kk = a.k > 0 ? a.k : 1;
+  if (!a.strided || a.k == 0) {
+    const int64_t total = a.rows * ((kk + 7) / 8);
+    digits_contig<CPLX, KD><<<(unsigned)((total + 255) / 256), 256, 0, st>>>(
+        a.X, a.ld, a.rows, a.k, a.conj, a.s, a.Kp, a.plane_rows, a.maxbits, a.exps, a.D, pr);
+  } else {
+    const dim3 grid((unsigned)((a.rows + 31) / 32), (unsigned)((a.k + 63) / 64));
+    digits_strided<CPLX, KD><<<grid, 256, 0, st>>>(a.X, a.ld, a.rows, a.k, a.conj, a.s, a.Kp, a.plane_rows, a.maxbits,
+                                                   a.exps, a.D, pr);
+  }
+  note_launch();
+}
+}  // namespace
+
 cudaError_t launch_digits(const SplitArgs& a, cudaStream_t st) {
   if (a.rows <= 0) return cudaSuccess;
-  const PlaneRange pr{a.plane_from, a.plane_to, a.gate};
-  int64_t kk = a.k > 0 ? a.k : 1;
-  if (!a.strided || a.k == 0) {
-    int64_t groups = (kk + 7) / 8;
-    int64_t total = a.rows * groups;
-    unsigned grid = (unsigned)((total + 255) / 256);
-    if (a.cplx)
-      { digits_contig<1><<<grid, 256, 0, st>>>(a.X, a.ld, a.rows, a.k, a.conj, a.s, a.Kp, a.plane_rows, a.maxbits,
-                                             a.exps, a.D, pr); note_launch(); }
-    else
-      { digits_contig<0><<<grid, 256, 0, st>>>(a.X, a.ld, a.rows, a.k, a.conj, a.s, a.Kp, a.plane_rows, a.maxbits,
-                                             a.exps, a.D, pr); note_launch(); }
+  if (a.cplx) {
+    if (a.kd) digits_launch<1, 1>(a, st);
+    else digits_launch<1, 0>(a, st);
   } else {
-    dim3 grid((unsigned)((a.rows + 31) / 32), (unsigned)((a.k + 63) / 64));
-    if (a.cplx)
-      { digits_strided<1><<<grid, 256, 0, st>>>(a.X, a.ld, a.rows, a.k, a.conj, a.s, a.Kp, a.plane_rows, a.maxbits,
-                                              a.exps, a.D, pr); note_launch(); }
-    else
-      { digits_strided<0><<<grid, 256, 0, st>>>(a.X, a.ld, a.rows, a.k, a.conj, a.s, a.Kp, a.plane_rows, a.maxbits,
-                                              a.exps, a.D, pr); note_launch(); }
+    if (a.kd) digits_launch<0, 1>(a, st);
+    else digits_launch<0, 0>(a, st);
   }
   return cudaGetLastError();
 }

@@ -6,6 +6,8 @@
 #include <cuda_fp16.h>
 #include <cstdint>
 
+#include "ozg_planes.h"
+
 namespace ozg {
 
 constexpr uint64_t kAbsMask = 0x7FFFFFFFFFFFFFFFull;
@@ -95,6 +97,52 @@ __device__ __forceinline__ void store_digit_planes(const DigitSrc (&d)[8], int t
 #pragma unroll
   for (int t = 1; t <= TMAX; ++t)
     if (t >= t_lo && t <= t_hi) *reinterpret_cast<uint4*>(out + (int64_t)(t - 1) * plane) = digits8(d, t);
+}
+
+// The same in a set with difference planes up to kd slices (kd_plane): digit planes t_lo .. t_hi.
+template <int TMAX>
+__device__ __forceinline__ void store_digit_planes_kd(const DigitSrc (&d)[8], int t_lo, int t_hi, __half* out,
+                                                      int64_t plane, int kd) {
+#pragma unroll
+  for (int t = 1; t <= TMAX; ++t)
+    if (t >= t_lo && t <= t_hi) *reinterpret_cast<uint4*>(out + (int64_t)kd_plane(t, kd) * plane) = digits8(d, t);
+}
+
+// Digit and difference planes of the blocks t_lo .. t_hi (t_hi <= TMAX) of eight consecutive
+// elements, in the order they are stored in.  1024 + |d| is FP16-exact, so one half2 subtraction
+// gives |d_p| - |d_q| (or the other way round when swapped), and the element's sign, which both
+// digits share, is XORed in.
+template <int TMAX>
+__device__ __forceinline__ void store_difference_planes(const DigitSrc (&d)[8], int t_lo, int t_hi, __half* out,
+                                                        int64_t plane, bool swapped) {
+  uint32_t m[TMAX][4], neg[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) neg[i] = d[2 * i].neg | (d[2 * i + 1].neg << 16);
+  auto diff = [&](uint32_t a, uint32_t b, int i) {
+    const __half2 v = __hsub2(*reinterpret_cast<const __half2*>(&a), *reinterpret_cast<const __half2*>(&b));
+    return *reinterpret_cast<const uint32_t*>(&v) ^ neg[i];
+  };
+#pragma unroll
+  for (int t = 1; t <= TMAX; ++t) {
+    if (t > t_hi) break;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) m[t - 1][i] = 0x64006400u | digit_mag(d[2 * i], t) | (digit_mag(d[2 * i + 1], t) << 16);
+#pragma unroll
+    for (int p = 0; p <= t / 2; ++p) {  // p = 0: the digit plane t; then p and q = t + 1 - p
+      uint4 o;
+      if (p == 0) {
+        o = make_uint4(diff(m[t - 1][0], 0x64006400u, 0), diff(m[t - 1][1], 0x64006400u, 1),
+                       diff(m[t - 1][2], 0x64006400u, 2), diff(m[t - 1][3], 0x64006400u, 3));
+      } else {
+        const uint32_t(&a)[4] = m[p > 0 ? p - 1 : 0];
+        const uint32_t(&b)[4] = m[t - p];
+        o = swapped ? make_uint4(diff(b[0], a[0], 0), diff(b[1], a[1], 1), diff(b[2], a[2], 2), diff(b[3], a[3], 3))
+                    : make_uint4(diff(a[0], b[0], 0), diff(a[1], b[1], 1), diff(a[2], b[2], 2), diff(a[3], b[3], 3));
+      }
+      if (t >= t_lo) *reinterpret_cast<uint4*>(out) = o;
+      out += plane;
+    }
+  }
 }
 
 }  // namespace ozg
