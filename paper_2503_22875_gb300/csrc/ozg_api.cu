@@ -48,7 +48,7 @@ int emu_gemm(ozg_ctx* c, bool cplx, char ta, char tb, int64_t m, int64_t n, int6
   if (autos) s = std::max(c->sel_s_hi, s_fb);
   const int nsamp = autos ? std::max(c->check_samples, 64) : c->check_samples;
   const bool beta_zero0 = (beta[0] == 0.0 && (!cplx || beta[1] == 0.0));
-  const int64_t Kp = (int64_t)align_up((size_t)k, 8);
+  const int64_t Kp = ozg::plane_pitch(k);
   const int64_t prA = cplx ? 2 * m : m, prB = cplx ? 2 * n : n;
   const int BM = ozg::slice_gemm_tile_m();
   auto grid_of = [&](int variant) {

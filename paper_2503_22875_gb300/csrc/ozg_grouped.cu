@@ -218,7 +218,7 @@ int build_plan(ozg_ctx* c, int64_t count, const ozg_gemm_desc* d, const std::vec
   P->oMax = max0;
   P->max_bytes = cv.off - max0;
   for (int64_t i = 0; i < count; ++i) {
-    const int64_t Kp = (d[i].k + 7) / 8 * 8;
+    const int64_t Kp = plane_pitch(d[i].k);
     oEA[i] = cv.take(4 * (size_t)d[i].m);
     oEB[i] = cv.take(4 * (size_t)d[i].n);
     oDA[i] = cv.take((size_t)planes[i] * d[i].m * Kp * 2);
@@ -303,7 +303,7 @@ int build_plan(ozg_ctx* c, int64_t count, const ozg_gemm_desc* d, const std::vec
   std::vector<CheckArgs> chk(count);
   int* flags = gat<int>(c, P->oFlags);
   for (int64_t i = 0; i < count; ++i) {
-    const int64_t Kp = (d[i].k + 7) / 8 * 8;
+    const int64_t Kp = plane_pitch(d[i].k);
     SplitArgs a;
     a.X = d[i].A;
     a.ld = d[i].lda;

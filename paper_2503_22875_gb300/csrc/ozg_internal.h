@@ -26,7 +26,7 @@ struct SplitArgs {
   int conj = 0;
   int cplx = 0;
   int s = 0;
-  int64_t Kp = 0;                 // row pitch of the digit planes (elements), multiple of 8, >= k
+  int64_t Kp = 0;                 // row pitch of the digit planes (elements; plane_pitch), multiple of 8, >= k
   int64_t plane_rows = 0;         // rows per digit plane (rows, or 2*rows for complex)
   __half* D = nullptr;            // digit planes [s][plane_rows][Kp], fp16 holding integers |d| <= 127
   unsigned long long* maxbits = nullptr;  // [rows] scratch, zeroed by the launcher
