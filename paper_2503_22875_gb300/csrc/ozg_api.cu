@@ -59,32 +59,41 @@ int emu_gemm(ozg_ctx* c, bool cplx, char ta, char tb, int64_t m, int64_t n, int6
   const int grid_kd = (int)std::min<int64_t>(2 * ozg::kd_tiles(prA, prB), c->num_sms / 2 * 2);
   // difference planes up to kd slices (0: none): a fixed count's own, or every learned count that
   // the difference-plane kernel takes
-  int kd = Gdbg ? 0 : choose_kd(c, cplx, prA, prB, k, autos ? std::min(c->sel_s_hi, ozg::kKdMax) : s, s);
-  int nplanes;
+  int variant = choose_variant(c, prA, prB, k, s);
+  SinglePlan plan;
+  if (!Gdbg) plan = plan_single(c, cplx, prA, prB, k, autos ? std::min(c->sel_s_hi, ozg::kKdMax) : s, s);
+  if (!plan.kd && variant != ozg::kStackedVariant) plan.parts = 1;
+  const int64_t tiles128 = ((prA + 127) / 128) * ((prB + 127) / 128);
+  int kd, nplanes;
   Carve cv;
-  size_t oDA, oDB, oE, oF, oMA, oMB, oR, oCold, oHist, oSd, oErr2, oSaved;
+  size_t oDA, oDB, oE, oF, oNf, oMA, oMB, oSplit, zero_end, oR, oCold, oHist, oSd, oErr2, oSaved;
   auto layout = [&]() {
+    kd = plan.kd;
     nplanes = ozg::kd_planes(s, kd);
     const int grid = std::max({grid_of(0), grid_of(1), kd ? grid_kd : 0});  // R scratch for every kernel
     cv = Carve();
     oDA = cv.take((size_t)nplanes * prA * Kp * 2), oDB = cv.take((size_t)nplanes * prB * Kp * 2);
     oE = cv.take(4 * (size_t)m), oF = cv.take(4 * (size_t)n);
+    // zeroed by one memset: the non-finite flag, the row maxima, the window sums of a split call
+    oNf = cv.take(sizeof(int));
     oMA = cv.take(8 * (size_t)m), oMB = cv.take(8 * (size_t)n);
+    oSplit = cv.take(plan.kd || plan.parts < 2 ? 0 : (size_t)tiles128 * plan.part_windows * 128 * 128 * 8);
+    zero_end = cv.off;
     oR = cv.take((size_t)grid * BM * 256 * 16);  // 16 bytes per output (128-bit Horner sum)
     oCold = cv.take((size_t)(nsamp > 0 ? nsamp : 1) * 16);
     oHist = cv.take(2 * 10 * 8), oSd = cv.take(4 * sizeof(int)), oErr2 = cv.take(sizeof(double));
     oSaved = cv.take((autos && !beta_zero0) ? (size_t)m * n * (cplx ? 16 : 8) : 8);
   };
   layout();
-  if (kd && !ws_available(c, cv.off)) {  // without the differences where the memory is not there
-    kd = 0;
+  if ((kd || plan.parts > 1) && !ws_available(c, cv.off)) {  // without either where the memory is not there
+    plan = SinglePlan();
     layout();
   }
   int rc = ensure_ws(c, cv.off);
   if (rc) return rc;
   cudaStream_t st = c->stream;
-  int* nonfinite = c->dflags + 1;
-  OZG_CUDA(cudaMemsetAsync(nonfinite, 0, sizeof(int), st));
+  int* nonfinite = at<int>(c, oNf);
+  OZG_CUDA(cudaMemsetAsync(nonfinite, 0, zero_end - oNf, st));
 
   PhaseScope* split_scope = new PhaseScope(c, OZG_PHASE_SPLIT);
   ozg::SplitArgs sa;
@@ -102,6 +111,7 @@ int emu_gemm(ozg_ctx* c, bool cplx, char ta, char tb, int64_t m, int64_t n, int6
   sa.maxbits = at<unsigned long long>(c, oMA);
   sa.exps = at<int32_t>(c, oE);
   sa.nonfinite = nonfinite;
+  sa.zeroed = 1;
   sa.kd = kd;
   sa.diff = 1;
   // learned count: row maxima -> features -> selection -> digits up to the selected count only
@@ -159,7 +169,7 @@ int emu_gemm(ozg_ctx* c, bool cplx, char ta, char tb, int64_t m, int64_t n, int6
   OZG_CUDA(ozg::make_digit_tmap(&tmB[0], sb.D, k, prB, Kp, nplanes, ozg::slice_gemm_tile_n_of(0), kd != 0));
   OZG_CUDA(ozg::make_digit_tmap(&tmB[1], sb.D, k, prB, Kp, nplanes, ozg::slice_gemm_tile_n_of(1), kd != 0));
   // tmB[v & 1] serves variant v
-  int variant = kd ? ozg::kStackedVariant : choose_variant(c, prA, prB, k, s);
+  if (kd) variant = ozg::kStackedVariant;
   ozg::GemmArgs ga;
   ga.rows = prA;
   ga.cols = prB;
@@ -263,7 +273,17 @@ int emu_gemm(ozg_ctx* c, bool cplx, char ta, char tb, int64_t m, int64_t n, int6
       OZG_CUDA(ozg::launch_slice_gemm_kd(tmA, tmB[1], gd, st));  // tmB[1]: boxes of 128 columns
     }
     // a learned count above kd runs on the digit planes alone
-    if (!kd || (autos && s > kd)) OZG_CUDA(ozg::launch_slice_gemm(tmA, tmB[ga.variant & 1], ga, st));
+    if (!kd || (autos && s > kd)) {
+      ozg::GemmArgs gp = ga;
+      if (!kd && plan.parts > 1 && ga.variant == ozg::kStackedVariant) {
+        gp.parts = plan.parts;
+        gp.part_kb = plan.part_kb;
+        gp.part_windows = plan.part_windows;
+        gp.Wsplit = at<unsigned long long>(c, oSplit);
+        gp.grid = (int)std::min<int64_t>(tiles128 * plan.parts, c->num_sms);
+      }
+      OZG_CUDA(ozg::launch_slice_gemm(tmA, tmB[gp.variant & 1], gp, st));
+    }
   }
   if (Gdbg) return OZG_OK;
 

@@ -635,7 +635,7 @@ __device__ __forceinline__ int stk_len0(int s, int win) {
 // the accumulator columns that collect the most
 __device__ __forceinline__ int stk_sweeps(int ga, bool two) { return stk::CHAIN_STAGES / (two ? ga : ga - 1); }
 
-template <bool GROUPED>
+template <bool GROUPED, bool SPLIT = false>
 __device__ __forceinline__ void stacked_body(const CUtensorMap* tmA0, const CUtensorMap* tmB0, const GemmArgs* P,
                                              const GroupArgs* G) {
   using namespace stk;
@@ -649,7 +649,9 @@ __device__ __forceinline__ void stacked_body(const CUtensorMap* tmA0, const CUte
 
   int* status = GROUPED ? G->status : P->status;
   double* Rws = GROUPED ? G->Rws : P->Rws;
-  const int ntiles = GROUPED ? G->ntiles : (int)(((P->rows + BM - 1) / BM) * ((P->cols + 127) / 128));
+  // SPLIT: a work item is one of P->parts ranges of P->part_kb 64-wide k sub-tiles of a tile
+  const int tiles = GROUPED ? G->ntiles : (int)(((P->rows + BM - 1) / BM) * ((P->cols + 127) / 128));
+  const int ntiles = SPLIT ? tiles * P->parts : tiles;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     for (int i = 0; i < NE; ++i) {
@@ -706,14 +708,15 @@ __device__ __forceinline__ void stacked_body(const CUtensorMap* tmA0, const CUte
             tnext += gridDim.x;
           }
           if (t < 0) break;
-          const TileJob j = get_job<128, 2, GROUPED>(t, tmA0, tmB0, P, G);
+          const TileJob j = get_job<128, 2, GROUPED>(SPLIT ? t % tiles : t, tmA0, tmB0, P, G);
           if (j.skip) continue;
           if (GROUPED && j.tmA != last_map) {
             tensormap_acquire(j.tmA);
             tensormap_acquire(j.tmB);
             last_map = j.tmA;
           }
-          const int KB = (j.KB - 1) * 2 + j.klast;  // 64-wide k sub-tiles
+          const int kb0 = SPLIT ? t / tiles * P->part_kb : 0;  // 64-wide k sub-tiles kb0 .. kb0 + KB - 1
+          const int KB = SPLIT ? min(P->part_kb, (j.KB - 1) * 2 + j.klast - kb0) : (j.KB - 1) * 2 + j.klast;
           const int arow = j.tm * BM, brow = j.tn * 128;
           const int win = window_len(j.s, (int64_t)j.KB * 128, j.cplx);
           int pc = 0;
@@ -724,7 +727,7 @@ __device__ __forceinline__ void stacked_body(const CUtensorMap* tmA0, const CUte
               bool two;
               stk_pass(wstart, wlen, q, ga, two);
               for (int kbi = 0; kbi < KB; ++kbi) {
-                const int kb = (pc & 1) ? KB - 1 - kbi : kbi;  // snake: a pass starts where the last ended
+                const int kb = kb0 + ((pc & 1) ? KB - 1 - kbi : kbi);  // snake: a pass starts where the last ended
                 const int kbn = (pc & 1) ? kb - 1 : kb + 1;    // the sweep's next k block
                 // stage i: A_i (i >= 1) and B_{ga-i} (i <= ga - 1); with two groups, stage ga also
                 // carries B_ga of the next k block, so only the pass's first sweep has a stage 0;
@@ -798,9 +801,9 @@ __device__ __forceinline__ void stacked_body(const CUtensorMap* tmA0, const CUte
             tnext += gridDim.x;
           }
           if (t < 0) break;
-          const TileJob j = get_job<128, 2, GROUPED>(t, tmA0, tmB0, P, G);
+          const TileJob j = get_job<128, 2, GROUPED>(SPLIT ? t % tiles : t, tmA0, tmB0, P, G);
           if (j.skip) continue;
-          const int KB = (j.KB - 1) * 2 + j.klast;
+          const int KB = SPLIT ? min(P->part_kb, (j.KB - 1) * 2 + j.klast - t / tiles * P->part_kb) : (j.KB - 1) * 2 + j.klast;
           const int win = window_len(j.s, (int64_t)j.KB * 128, j.cplx);
           for (int wstart = 2, wlen = stk_len0(j.s, win); wstart <= j.s + 1;
                wstart += wlen, wlen = min(win, j.s + 2 - wstart)) {
@@ -924,10 +927,10 @@ __device__ __forceinline__ void stacked_body(const CUtensorMap* tmA0, const CUte
         tnext += gridDim.x;
       }
       if (t < 0) break;
-      const TileJob j = get_job<128, 2, GROUPED>(t, tmA0, tmB0, P, G);
+      const TileJob j = get_job<128, 2, GROUPED>(SPLIT ? t % tiles : t, tmA0, tmB0, P, G);
       if (j.skip) continue;
       const int s = j.s;
-      const int KB = (j.KB - 1) * 2 + j.klast;
+      const int KB = SPLIT ? min(P->part_kb, (j.KB - 1) * 2 + j.klast - t / tiles * P->part_kb) : (j.KB - 1) * 2 + j.klast;
       const int64_t grow = (int64_t)j.tm * BM + r;
       const bool row_ok = grow < j.rows;
       const int64_t orow = j.cplx ? (grow >> 1) : grow;
@@ -971,7 +974,7 @@ __device__ __forceinline__ void stacked_body(const CUtensorMap* tmA0, const CUte
 #pragma unroll
         for (int c = 0; c < NOUT; ++c) W[c] = 0;
         long long* sbuf = reinterpret_cast<long long*>(smem + S0_OFF) + ew * 32 + lane;
-        if (widx >= 1 && nfin > 0) {  // the first chunk's spilled words, staged while this window drains
+        if (!SPLIT && widx >= 1 && nfin > 0) {  // the first chunk's spilled words, staged while this window drains
 #pragma unroll
           for (int i = 0; i < 8; ++i) cp_async8(sbuf + i * EPI_WARPS * 32, pa.S0 + (size_t)i * BM);
           cp_async_commit();
@@ -1041,6 +1044,15 @@ __device__ __forceinline__ void stacked_body(const CUtensorMap* tmA0, const CUte
             acc_par ^= 1u << buf;
             buf ^= 1;
           }
+        }
+        if (SPLIT) {
+          // this k range's share of the window: added to the tile's words (the finish kernel rounds)
+          unsigned long long* Wt = P->Wsplit + ((size_t)(t % tiles) * P->part_windows + widx) * BM * 128 +
+                                   (size_t)(j.cplx ? chalf * NOUT / 2 : chalf * NOUT) * BM + r;
+#pragma unroll
+          for (int c = 0; c < NOUT; ++c)
+            if (c < nfin) atomicAdd(Wt + (size_t)c * BM, (unsigned long long)W[c]);
+          continue;
         }
         // the window is complete: spill the first one, close a later one into the FP64
         // partial, or round the last one and write C (chunks of 8 outputs, the array rotated
@@ -1122,6 +1134,58 @@ __global__ void __launch_bounds__(THREADS, 1)
   if (P.nonfinite != nullptr && *P.nonfinite) return;
   if (P.kd != 0 && P.s_dev != nullptr && *P.s_dev <= P.kd) return;  // the difference-plane launch runs
   stacked_body<false>(&tmA, &tmB, &P, nullptr);
+}
+// The same with every tile's k range cut into parts, each part a work item of its own.
+__global__ void __launch_bounds__(THREADS, 1)
+    slice_gemm_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
+                            const GemmArgs P) {
+  if (P.nonfinite != nullptr && *P.nonfinite) return;
+  if (P.kd != 0 && P.s_dev != nullptr && *P.s_dev <= P.kd) return;
+  stacked_body<false, true>(&tmA, &tmB, &P, nullptr);
+}
+// Rounds the window sums of the split kernel and writes C: a block per tile and chunk of 8 outputs,
+// a thread per row.  HBM / L2 bound: 8 bytes read per output and window.
+__global__ void __launch_bounds__(BM) split_finish_kernel(const GemmArgs P) {
+  if (P.nonfinite != nullptr && *P.nonfinite) return;
+  if (P.kd != 0 && P.s_dev != nullptr && *P.s_dev <= P.kd) return;
+  const int chunks = P.cplx ? 8 : 16;
+  TileJob j = get_job<128, 2, false>((int)(blockIdx.x / chunks), nullptr, nullptr, &P, nullptr);
+  const int o = (int)(blockIdx.x % chunks) * 8, r = threadIdx.x;
+  const int win = window_len(j.s, (int64_t)j.KB * 128, j.cplx);
+  const int64_t grow = (int64_t)j.tm * BM + r;
+  PushArgs pa;
+  pa.orow = j.cplx ? (grow >> 1) : grow;
+  pa.row_ok = grow < j.rows;
+  pa.gcol0 = (int64_t)j.tn * 128;
+  pa.unit_ab = j.beta_zero && j.a0 == 1.0 && j.a1 == 0.0;
+  pa.odd = (r & 1) != 0;
+  pa.ebase = (pa.row_ok ? j.e[pa.orow] : 0) - 7 * (j.s + 1);
+  pa.kind = kFinal;
+  const long long* Wt =
+      reinterpret_cast<const long long*>(P.Wsplit) + (size_t)(blockIdx.x / chunks) * P.part_windows * BM * 128 + (size_t)o * BM + r;
+  const int64_t c0 = (j.cplx ? (pa.gcol0 >> 1) : pa.gcol0) + o, climit = j.cplx ? j.n : j.cols;
+  if (c0 >= climit) return;
+  long long s0[8], rw[8];
+  int fe[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    rw[i] = __ldcg(Wt + (size_t)i * BM);
+    fe[i] = c0 + i < climit ? __ldg(j.f + c0 + i) : 0;
+    s0[i] = 0;
+  }
+  int widx = 0, wstart = 2, wlen = stk_len0(j.s, win);
+  for (; wstart + wlen <= j.s + 1; ++widx) {  // the last window's words end in rw, the earlier ones' in s0
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      s0[i] = widx == 0 ? rw[i] : close_val(s0[i], rw[i], widx, wlen);
+      rw[i] = __ldcg(Wt + (size_t)(widx + 1) * BM * 128 + (size_t)i * BM);
+    }
+    wstart += wlen;
+    wlen = min(win, j.s + 2 - wstart);
+  }
+  pa.widx = widx;
+  pa.wlen = wlen;
+  window_out<8, false, true>(rw, o, pa, j, s0, fe);
 }
 __global__ void __launch_bounds__(THREADS, 1) slice_gemm_grouped_stacked_kernel(const GroupArgs G) {
   if (G.run != nullptr && *G.run == 0) return;
@@ -1262,6 +1326,9 @@ cudaError_t prepare_kernels() {
   if ((e = cudaFuncSetAttribute(slice_gemm_stacked_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)stk::SMEM)) != cudaSuccess)
     return e;
+  if ((e = cudaFuncSetAttribute(slice_gemm_split_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)stk::SMEM)) != cudaSuccess)
+    return e;
   if ((e = cudaFuncSetAttribute(slice_gemm_grouped_stacked_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)stk::SMEM)) != cudaSuccess)
     return e;
@@ -1286,6 +1353,16 @@ cudaError_t prepare_kernels() {
 
 cudaError_t launch_slice_gemm(const CUtensorMap& tmA, const CUtensorMap& tmB, const GemmArgs& a, cudaStream_t st) {
   if (a.grid <= 0) return cudaSuccess;
+  if (a.parts > 1) {
+    if (a.variant != kStackedVariant || a.exact || a.Gdbg != nullptr || a.s > stacked_max_slices())
+      return cudaErrorInvalidValue;
+    slice_gemm_split_kernel<<<a.grid, THREADS, stk::SMEM, st>>>(tmA, tmB, a);
+    note_launch();
+    const int64_t tiles = ((a.rows + BM - 1) / BM) * ((a.cols + 127) / 128);
+    split_finish_kernel<<<(unsigned)(tiles * (a.cplx ? 8 : 16)), BM, 0, st>>>(a);
+    note_launch();
+    return cudaGetLastError();
+  }
   // a plane set with differences is read by the stacked kernel only
   if (a.kd != 0 && (a.variant != kStackedVariant || a.exact || a.Gdbg != nullptr || a.s > stacked_max_slices()))
     return cudaErrorInvalidValue;

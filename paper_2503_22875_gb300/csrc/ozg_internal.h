@@ -39,6 +39,7 @@ struct SplitArgs {
   const int* plane_to = nullptr;
   const int* gate = nullptr;
   int kd = 0;    // plane layout: difference planes up to this slice count (0: digit planes only)
+  int zeroed = 0;  // maxbits is zero already
   int diff = 0;  // +1: write the differences digit p - digit q, -1: digit q - digit p, 0: none; they
                  // are written when t_hi <= kd
 };
@@ -74,6 +75,10 @@ struct GemmArgs {
   int defer = 0;                // 1: spread intermediate epilogue pushes over the next drains
   const int* s_dev = nullptr;   // if set, the slice count is read here (device-chosen); s = plane count
   int exact = 0;                // 1: exact 128-bit Horner sum and one rounding (s <= 13)
+  // stacked kernel: every tile's k range cut into `parts` of part_kb 64-wide sub-tiles, whose window
+  // sums meet in Wsplit ([tile][part_windows][128][128] words, zero before the launch)
+  int parts = 1, part_kb = 0, part_windows = 0;
+  unsigned long long* Wsplit = nullptr;
   int kd = 0;                   // difference planes: the planes' layout is kd_plane's for this count
 };
 

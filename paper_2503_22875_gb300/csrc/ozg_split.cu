@@ -217,8 +217,10 @@ __global__ void digits_to_i8(const __half* __restrict__ D, int64_t planes_rows, 
 
 cudaError_t launch_rowmax(const SplitArgs& a, cudaStream_t st) {
   if (a.rows <= 0) return cudaSuccess;
-  cudaError_t err = cudaMemsetAsync(a.maxbits, 0, sizeof(unsigned long long) * a.rows, st);
-  if (err != cudaSuccess) return err;
+  if (!a.zeroed) {
+    cudaError_t err = cudaMemsetAsync(a.maxbits, 0, sizeof(unsigned long long) * a.rows, st);
+    if (err != cudaSuccess) return err;
+  }
   if (a.k > 0) {
     if (!a.strided) {
       int wpb = 8;
