@@ -314,6 +314,7 @@ __global__ void __launch_bounds__(kStatsThreads, 3) stats_batched(const SplitArg
 // The two operands of one call, passed by value (single calls need no device job table).
 template <bool HIST>
 __global__ void __launch_bounds__(kStatsThreads, 3) stats_pair(const SplitArgs a, const SplitArgs b, int64_t units_a) {
+  pdl_entry();
   const bool first = (int64_t)blockIdx.x < units_a;
   stats_unit<HIST>(first ? a : b, first ? (int64_t)blockIdx.x : (int64_t)blockIdx.x - units_a);
 }
@@ -592,10 +593,9 @@ cudaError_t launch_stats_pair(const SplitArgs& a, const SplitArgs& b, cudaStream
   const int64_t ua = stats_units_of(a), ub = stats_units_of(b);
   if (ua + ub <= 0) return cudaSuccess;
   if (a.hist != nullptr || b.hist != nullptr)
-    stats_pair<true><<<(unsigned)(ua + ub), kStatsThreads, kStatsHistSmem, st>>>(a, b, ua);
+    launch_pdl(stats_pair<true>, (unsigned)(ua + ub), kStatsThreads, kStatsHistSmem, st, a, b, ua);
   else
-    stats_pair<false><<<(unsigned)(ua + ub), kStatsThreads, 0, st>>>(a, b, ua);
-  note_launch();
+    launch_pdl(stats_pair<false>, (unsigned)(ua + ub), kStatsThreads, 0, st, a, b, ua);
   return cudaGetLastError();
 }
 

@@ -51,6 +51,7 @@ __device__ __forceinline__ double ld_op(const double* X, int64_t ld, char t, int
 __device__ void check_one(const CheckArgs& P, int sample, int lane, double* err_slot);
 
 __global__ void check_pre(CheckArgs P) {
+  pdl_entry();
   if (P.gate != nullptr && *P.gate) return;
   int idx = blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= P.nsamp) return;
@@ -191,6 +192,7 @@ __device__ void check_one(const CheckArgs& P, int sample, int lane, double* err_
 }
 
 __global__ void check_post(CheckArgs P) {
+  pdl_entry();
   if (P.gate != nullptr && *P.gate) return;
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (warp >= P.nsamp) return;
@@ -228,14 +230,15 @@ __global__ void check_post_batched(const CheckArgs* calls, int ncalls, int nsamp
 
 cudaError_t launch_check_pre(const CheckArgs& a, cudaStream_t st) {
   if (a.nsamp <= 0 || a.beta_zero) return cudaSuccess;
-  { check_pre<<<(a.nsamp + 127) / 128, 128, 0, st>>>(a); note_launch(); }
+  launch_pdl(check_pre, (a.nsamp + 127) / 128, 128, 0, st, a);
   return cudaGetLastError();
 }
 
 cudaError_t launch_check_batched_pre(const CheckArgs* calls_dev, int ncalls, int nsamp, cudaStream_t st) {
   const int64_t total = (int64_t)ncalls * nsamp;
   if (total <= 0) return cudaSuccess;
-  { check_pre_batched<<<(unsigned)((total + 127) / 128), 128, 0, st>>>(calls_dev, ncalls, nsamp); note_launch(); }
+  check_pre_batched<<<(unsigned)((total + 127) / 128), 128, 0, st>>>(calls_dev, ncalls, nsamp);
+  note_launch();
   return cudaGetLastError();
 }
 
@@ -245,7 +248,8 @@ cudaError_t launch_check_batched_post(const CheckArgs* calls_dev, int ncalls, in
   if (total <= 0) return cudaSuccess;
   cudaError_t e = cudaMemsetAsync(errs_dev, 0, sizeof(double) * ncalls, st);
   if (e != cudaSuccess) return e;
-  { check_post_batched<<<(unsigned)((total + 3) / 4), 128, 0, st>>>(calls_dev, ncalls, nsamp); note_launch(); }
+  check_post_batched<<<(unsigned)((total + 3) / 4), 128, 0, st>>>(calls_dev, ncalls, nsamp);
+  note_launch();
   return cudaGetLastError();
 }
 
@@ -255,7 +259,7 @@ cudaError_t launch_check_post(const CheckArgs& a, cudaStream_t st) {
   if (e == cudaSuccess && a.part_err != nullptr) e = cudaMemsetAsync(a.part_err, 0, 2 * sizeof(double), st);
   if (e != cudaSuccess) return e;
   const int warps_per_block = 4;
-  { check_post<<<(a.nsamp + warps_per_block - 1) / warps_per_block, 32 * warps_per_block, 0, st>>>(a); note_launch(); }
+  launch_pdl(check_post, (a.nsamp + warps_per_block - 1) / warps_per_block, 32 * warps_per_block, 0, st, a);
   return cudaGetLastError();
 }
 

@@ -1110,6 +1110,7 @@ template <int BN_, int SUB_>
 __global__ void __launch_bounds__(THREADS, 1)
     slice_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                       const GemmArgs P) {
+  pdl_entry();
   if (P.nonfinite != nullptr && *P.nonfinite) return;  // the native FP64 kernel handles this call
   gemm_body<BN_, SUB_, false>(&tmA, &tmB, &P, nullptr);
 }
@@ -1131,6 +1132,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1) slice_ge
 __global__ void __launch_bounds__(THREADS, 1)
     slice_gemm_stacked_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                               const GemmArgs P) {
+  pdl_entry();
   if (P.nonfinite != nullptr && *P.nonfinite) return;
   if (P.kd != 0 && P.s_dev != nullptr && *P.s_dev <= P.kd) return;  // the difference-plane launch runs
   stacked_body<false>(&tmA, &tmB, &P, nullptr);
@@ -1139,6 +1141,7 @@ __global__ void __launch_bounds__(THREADS, 1)
 __global__ void __launch_bounds__(THREADS, 1)
     slice_gemm_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                             const GemmArgs P) {
+  pdl_entry();
   if (P.nonfinite != nullptr && *P.nonfinite) return;
   if (P.kd != 0 && P.s_dev != nullptr && *P.s_dev <= P.kd) return;
   stacked_body<false, true>(&tmA, &tmB, &P, nullptr);
@@ -1146,6 +1149,7 @@ __global__ void __launch_bounds__(THREADS, 1)
 // Rounds the window sums of the split kernel and writes C: a block per tile and chunk of 8 outputs,
 // a thread per row.  HBM / L2 bound: 8 bytes read per output and window.
 __global__ void __launch_bounds__(BM) split_finish_kernel(const GemmArgs P) {
+  pdl_entry();
   if (P.nonfinite != nullptr && *P.nonfinite) return;
   if (P.kd != 0 && P.s_dev != nullptr && *P.s_dev <= P.kd) return;
   const int chunks = P.cplx ? 8 : 16;
@@ -1284,10 +1288,11 @@ cudaError_t launch_one(const CUtensorMap* tmA, const CUtensorMap* tmB, const Gem
   cudaError_t e;
   if (GROUPED) {
     if ((e = set_smem_once(slice_gemm_grouped_kernel<BN_, SUB_>, K::SMEM, done)) != cudaSuccess) return e;
-    { slice_gemm_grouped_kernel<BN_, SUB_><<<grid, THREADS, K::SMEM, st>>>(*g); note_launch(); }
+    slice_gemm_grouped_kernel<BN_, SUB_><<<grid, THREADS, K::SMEM, st>>>(*g);
+    note_launch();
   } else {
     if ((e = set_smem_once(slice_gemm_kernel<BN_, SUB_>, K::SMEM, done)) != cudaSuccess) return e;
-    { slice_gemm_kernel<BN_, SUB_><<<grid, THREADS, K::SMEM, st>>>(*tmA, *tmB, *a); note_launch(); }
+    launch_pdl(slice_gemm_kernel<BN_, SUB_>, grid, THREADS, K::SMEM, st, *tmA, *tmB, *a);
   }
   return cudaGetLastError();
 }
@@ -1299,11 +1304,11 @@ cudaError_t launch_stacked(const CUtensorMap* tmA, const CUtensorMap* tmB, const
   if (GROUPED) {
     if ((e = set_smem_once(slice_gemm_grouped_stacked_kernel, stk::SMEM, done)) != cudaSuccess) return e;
     slice_gemm_grouped_stacked_kernel<<<grid, THREADS, stk::SMEM, st>>>(*g);
+    note_launch();
   } else {
     if ((e = set_smem_once(slice_gemm_stacked_kernel, stk::SMEM, done)) != cudaSuccess) return e;
-    slice_gemm_stacked_kernel<<<grid, THREADS, stk::SMEM, st>>>(*tmA, *tmB, *a);
+    launch_pdl(slice_gemm_stacked_kernel, grid, THREADS, stk::SMEM, st, *tmA, *tmB, *a);
   }
-  note_launch();
   return cudaGetLastError();
 }
 template <bool GROUPED>
@@ -1356,11 +1361,9 @@ cudaError_t launch_slice_gemm(const CUtensorMap& tmA, const CUtensorMap& tmB, co
   if (a.parts > 1) {
     if (a.variant != kStackedVariant || a.exact || a.Gdbg != nullptr || a.s > stacked_max_slices())
       return cudaErrorInvalidValue;
-    slice_gemm_split_kernel<<<a.grid, THREADS, stk::SMEM, st>>>(tmA, tmB, a);
-    note_launch();
+    launch_pdl(slice_gemm_split_kernel, a.grid, THREADS, stk::SMEM, st, tmA, tmB, a);
     const int64_t tiles = ((a.rows + BM - 1) / BM) * ((a.cols + 127) / 128);
-    split_finish_kernel<<<(unsigned)(tiles * (a.cplx ? 8 : 16)), BM, 0, st>>>(a);
-    note_launch();
+    launch_pdl(split_finish_kernel, (unsigned)(tiles * (a.cplx ? 8 : 16)), BM, 0, st, a);
     return cudaGetLastError();
   }
   // a plane set with differences is read by the stacked kernel only

@@ -554,6 +554,7 @@ template <bool CPLX>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
     slice_gemm_kd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                          const GemmArgs P) {
+  pdl_entry();
   if (P.nonfinite != nullptr && *P.nonfinite) return;
   if (P.s_dev != nullptr && *P.s_dev > P.kd) return;  // no difference planes: the plane-by-plane launch runs
   kd_body<false, CPLX>(&tmA, &tmB, &P, nullptr);
@@ -574,10 +575,9 @@ cudaError_t launch_slice_gemm_kd(const CUtensorMap& tmA, const CUtensorMap& tmB,
   if (a.grid <= 0) return cudaSuccess;
   if (a.grid % 2) return cudaErrorInvalidValue;  // whole clusters
   if (a.cplx)
-    slice_gemm_kd_kernel<true><<<a.grid, THREADS, kd::SMEM, st>>>(tmA, tmB, a);
+    launch_pdl(slice_gemm_kd_kernel<true>, a.grid, THREADS, kd::SMEM, st, tmA, tmB, a);
   else
-    slice_gemm_kd_kernel<false><<<a.grid, THREADS, kd::SMEM, st>>>(tmA, tmB, a);
-  note_launch();
+    launch_pdl(slice_gemm_kd_kernel<false>, a.grid, THREADS, kd::SMEM, st, tmA, tmB, a);
   return cudaGetLastError();
 }
 

@@ -17,6 +17,34 @@ namespace ozg {
 long long& launch_counter();
 inline void note_launch() { __atomic_fetch_add(&launch_counter(), 1LL, __ATOMIC_RELAXED); }
 
+// The launches of a single call are programmatic dependents: a kernel is launched once every CTA of
+// its predecessor in the stream has started, and waits in pdl_entry, before its first access to
+// memory, until the predecessor has completed and its writes are visible.  Every kernel launched so
+// starts with pdl_entry in every thread, so the wait carries through the sequence (256^3 s = 7: 53.2
+// -> 40.9 us, complex 768^3 s = 6: 112 -> 100).  The batched kernels are launched plainly: they gained
+// nothing as dependents inside a graph, and beside other streams' work (the parts of a batch in host
+// memory) their waiting CTAs held SMs (2.98 -> 3.28 ms).
+#ifdef __CUDACC__
+__device__ __forceinline__ void pdl_entry() {
+  asm volatile("griddepcontrol.launch_dependents;\n griddepcontrol.wait;" ::: "memory");
+}
+template <typename... P, typename... A>
+void launch_pdl(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, const A&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kern, P(args)...);
+  note_launch();
+}
+#endif
+
 struct SplitArgs {
   const double* X = nullptr;
   int64_t ld = 0;

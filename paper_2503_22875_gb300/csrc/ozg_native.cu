@@ -42,6 +42,7 @@ __device__ __forceinline__ double2 zero_of(double2) { return make_double2(0.0, 0
 
 template <int CPLX>
 __global__ void __launch_bounds__(256) native_gemm_kernel(NativeArgs P) {
+  pdl_entry();
   using T = typename Elem<CPLX>::T;
   if (P.gate != nullptr && *P.gate == 0) return;
   __shared__ T As[TK][TM + 1];
@@ -150,9 +151,9 @@ cudaError_t launch_native_gemm(const NativeArgs& a, cudaStream_t st) {
   dim3 grid((unsigned)((a.n + TN - 1) / TN), (unsigned)((a.m + TM - 1) / TM));
   if (grid.y > 65535) return cudaErrorInvalidValue;
   if (a.cplx)
-    { native_gemm_kernel<1><<<grid, 256, 0, st>>>(a); note_launch(); }
+    launch_pdl(native_gemm_kernel<1>, grid, 256, 0, st, a);
   else
-    { native_gemm_kernel<0><<<grid, 256, 0, st>>>(a); note_launch(); }
+    launch_pdl(native_gemm_kernel<0>, grid, 256, 0, st, a);
   return cudaGetLastError();
 }
 

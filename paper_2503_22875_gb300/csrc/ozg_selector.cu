@@ -68,6 +68,7 @@ __device__ void hist_tile(const SplitArgs& J, int64_t u, unsigned int* sh) {
 }
 
 __global__ void __launch_bounds__(256) gap_hist_pair(SplitArgs a, SplitArgs b, int64_t units_a) {
+  pdl_entry();
   __shared__ unsigned int sh[10];
   if (threadIdx.x < 10) sh[threadIdx.x] = 0;
   __syncthreads();
@@ -215,6 +216,7 @@ __device__ void select_warp(const SelectorDev* M, const unsigned long long* hA, 
 __global__ void select_single(const SelectorDev* M, const unsigned long long* hA, const unsigned long long* hB,
                               int64_t m, int64_t n, int64_t k, float log10_target, int s_cap, int* s_out,
                               float* feat_out, float* prob_out) {
+  pdl_entry();
   select_warp(M, hA, hB, m, n, k, log10_target, s_cap, s_out, nullptr, feat_out, prob_out);
 }
 
@@ -310,6 +312,7 @@ __global__ void adam_kernel(float* theta, const float* grad, float* m1, float* m
 
 __global__ void repair_prep_kernel(const double* err, double target, int* not_repaired, const double* saved,
                                    double* C, int64_t m, int64_t n, int64_t ldc, int w, int restore) {
+  pdl_entry();
   const double e = *err;
   const bool bad = !(e <= target);  // NaN counts as a failed check
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -325,8 +328,8 @@ __global__ void repair_prep_kernel(const double* err, double target, int* not_re
 cudaError_t launch_repair_prep(const double* err, double target, int* not_repaired, const double* saved, double* C,
                                int64_t m, int64_t n, int64_t ldc, int w, int restore, cudaStream_t st) {
   const int64_t total = restore ? m * n * w : 1;
-  { repair_prep_kernel<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(err, target, not_repaired, saved, C, m, n, ldc, w,
-                                                                     restore); note_launch(); }
+  launch_pdl(repair_prep_kernel, (unsigned)((total + 255) / 256), 256, 0, st, err, target, not_repaired, saved, C, m, n, ldc, w,
+                                                                     restore);
   return cudaGetLastError();
 }
 
@@ -350,28 +353,30 @@ cudaError_t launch_adam(float* theta, const float* grad, float* m1, float* m2, i
 cudaError_t launch_gap_hist_pair(const SplitArgs& a, const SplitArgs& b, cudaStream_t st) {
   const int64_t ua = ((a.rows + 31) / 32) * ((a.k + 63) / 64), ub = ((b.rows + 31) / 32) * ((b.k + 63) / 64);
   if (ua + ub <= 0) return cudaSuccess;
-  { gap_hist_pair<<<(unsigned)(ua + ub), 256, 0, st>>>(a, b, ua); note_launch(); }
+  launch_pdl(gap_hist_pair, (unsigned)(ua + ub), 256, 0, st, a, b, ua);
   return cudaGetLastError();
 }
 
 cudaError_t launch_gap_hist_batched(const SplitArgs* jobs_dev, const int2* rowmax_units_dev, int64_t units,
                                     cudaStream_t st) {
   if (units <= 0) return cudaSuccess;
-  { gap_hist_batched<<<(unsigned)units, 256, 0, st>>>(jobs_dev, rowmax_units_dev); note_launch(); }
+  gap_hist_batched<<<(unsigned)units, 256, 0, st>>>(jobs_dev, rowmax_units_dev);
+  note_launch();
   return cudaGetLastError();
 }
 
 cudaError_t launch_select_single(const SelectorDev* M, const unsigned long long* hA, const unsigned long long* hB,
                                  int64_t m, int64_t n, int64_t k, float log10_target, int s_cap, int* s_out,
                                  float* feat_out, float* prob_out, cudaStream_t st) {
-  { select_single<<<1, 32, 0, st>>>(M, hA, hB, m, n, k, log10_target, s_cap, s_out, feat_out, prob_out); note_launch(); }
+  launch_pdl(select_single, 1, 32, 0, st, M, hA, hB, m, n, k, log10_target, s_cap, s_out, feat_out, prob_out);
   return cudaGetLastError();
 }
 
 cudaError_t launch_select_batched(const SelectorDev* M, const SelectJob* jobs_dev, int njobs, float log10_target,
                                   cudaStream_t st) {
   if (njobs <= 0) return cudaSuccess;
-  { select_batched<<<(njobs + 3) / 4, 128, 0, st>>>(M, jobs_dev, njobs, log10_target); note_launch(); }
+  select_batched<<<(njobs + 3) / 4, 128, 0, st>>>(M, jobs_dev, njobs, log10_target);
+  note_launch();
   return cudaGetLastError();
 }
 

@@ -62,6 +62,7 @@ __device__ __forceinline__ void flag_nonfinite(uint64_t absbits, int* nonfinite)
 // one warp per row; lanes stride along l
 __global__ void rowmax_contig(const double* __restrict__ X, int64_t ld, int64_t rows, int64_t k, int cplx,
                               unsigned long long* __restrict__ maxbits, int* nonfinite) {
+  pdl_entry();
   int64_t row = (int64_t)blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
   int lane = threadIdx.x % 32;
   if (row >= rows) return;
@@ -96,6 +97,7 @@ __global__ void rowmax_contig(const double* __restrict__ X, int64_t ld, int64_t 
 // thread per row (consecutive rows are contiguous in memory), grid.y splits k; atomicMax merges
 __global__ void rowmax_strided(const double* __restrict__ X, int64_t ld, int64_t rows, int64_t k, int64_t kchunk,
                                int cplx, unsigned long long* __restrict__ maxbits, int* nonfinite) {
+  pdl_entry();
   int64_t row = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (row >= rows) return;
   int64_t l0 = (int64_t)blockIdx.y * kchunk, l1 = min(k, l0 + kchunk);
@@ -127,6 +129,7 @@ template <int CPLX, int KD>
 __global__ void digits_contig(const double* __restrict__ X, int64_t ld, int64_t rows, int64_t k, int conj, int s,
                               int64_t Kp, int64_t plane_rows, const unsigned long long* __restrict__ maxbits,
                               int32_t* __restrict__ exps, __half* __restrict__ D, PlaneRange pr) {
+  pdl_entry();
   int t_lo, t_hi;
   if (!pr.resolve(s, t_lo, t_hi)) return;
   int64_t groups = (k + 7) / 8;
@@ -163,6 +166,7 @@ __global__ void __launch_bounds__(256) digits_strided(const double* __restrict__
                                                       const unsigned long long* __restrict__ maxbits,
                                                       int32_t* __restrict__ exps, __half* __restrict__ D,
                                                       PlaneRange pr) {
+  pdl_entry();
   int t_lo, t_hi;
   if (!pr.resolve(s, t_lo, t_hi)) return;
   constexpr int TR = 32, TL = 64;
@@ -225,7 +229,7 @@ cudaError_t launch_rowmax(const SplitArgs& a, cudaStream_t st) {
     if (!a.strided) {
       int wpb = 8;
       unsigned grid = (unsigned)((a.rows + wpb - 1) / wpb);
-      { rowmax_contig<<<grid, 32 * wpb, 0, st>>>(a.X, a.ld, a.rows, a.k, a.cplx, a.maxbits, a.nonfinite); note_launch(); }
+      launch_pdl(rowmax_contig, grid, 32 * wpb, 0, st, a.X, a.ld, a.rows, a.k, a.cplx, a.maxbits, a.nonfinite);
     } else {
       int64_t rb = (a.rows + 255) / 256;
       int64_t ksplit = (608 + rb - 1) / rb;  // ~4 CTAs per SM in total
@@ -234,8 +238,8 @@ cudaError_t launch_rowmax(const SplitArgs& a, cudaStream_t st) {
       if (ksplit < 1) ksplit = 1;
       int64_t kchunk = (a.k + ksplit - 1) / ksplit;
       ksplit = (a.k + kchunk - 1) / kchunk;
-      { rowmax_strided<<<dim3((unsigned)rb, (unsigned)ksplit), 256, 0, st>>>(a.X, a.ld, a.rows, a.k, kchunk, a.cplx,
-                                                                           a.maxbits, a.nonfinite); note_launch(); }
+      launch_pdl(rowmax_strided, dim3((unsigned)rb, (unsigned)ksplit), 256, 0, st, a.X, a.ld, a.rows, a.k, kchunk, a.cplx,
+                                                                           a.maxbits, a.nonfinite);
     }
   }
   return cudaGetLastError();
@@ -248,14 +252,13 @@ void digits_launch(const SplitArgs& a, cudaStream_t st) {
   const int64_t kk = a.k > 0 ? a.k : 1;
   if (!a.strided || a.k == 0) {
     const int64_t total = a.rows * ((kk + 7) / 8);
-    digits_contig<CPLX, KD><<<(unsigned)((total + 255) / 256), 256, 0, st>>>(
+    launch_pdl(digits_contig<CPLX, KD>, (unsigned)((total + 255) / 256), 256, 0, st, 
         a.X, a.ld, a.rows, a.k, a.conj, a.s, a.Kp, a.plane_rows, a.maxbits, a.exps, a.D, pr);
   } else {
     const dim3 grid((unsigned)((a.rows + 31) / 32), (unsigned)((a.k + 63) / 64));
-    digits_strided<CPLX, KD><<<grid, 256, 0, st>>>(a.X, a.ld, a.rows, a.k, a.conj, a.s, a.Kp, a.plane_rows, a.maxbits,
+    launch_pdl(digits_strided<CPLX, KD>, grid, 256, 0, st, a.X, a.ld, a.rows, a.k, a.conj, a.s, a.Kp, a.plane_rows, a.maxbits,
                                                    a.exps, a.D, pr);
   }
-  note_launch();
 }
 }  // namespace
 

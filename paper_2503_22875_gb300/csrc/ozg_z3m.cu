@@ -24,6 +24,7 @@ namespace {
 __global__ void __launch_bounds__(256) z3m_split_kernel(const double* __restrict__ X, int64_t rows, int64_t cols,
                                                         int64_t ld, int conj, double* __restrict__ Xr,
                                                         double* __restrict__ Xi, double* __restrict__ Xs) {
+  pdl_entry();
   const int64_t total = rows * cols;
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
     const int64_t i = t % rows, j = t / rows;
@@ -39,6 +40,7 @@ __global__ void __launch_bounds__(256) z3m_combine_kernel(const double* __restri
                                                           const double* __restrict__ P3, int64_t m, int64_t n,
                                                           double a0, double a1, double b0, double b1, int beta_zero,
                                                           double* C, int64_t ldc) {
+  pdl_entry();
   const int64_t total = m * n;
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
     const int64_t i = t % m, j = t / m;
@@ -112,8 +114,8 @@ extern "C" int ozg_zgemm3m(ozg_ctx* c, char transa, char transb, int64_t m, int6
   double *P2 = P1 + m * n, *P3 = P2 + m * n;
   {
     PhaseScope ps(c, OZG_PHASE_SPLIT);
-    { ozg::z3m_split_kernel<<<ozg::grid_for(c, ra * ca), 256, 0, st>>>(A, ra, ca, lda, ta == 'C', Ar, Ai, As); ozg::note_launch(); }
-    { ozg::z3m_split_kernel<<<ozg::grid_for(c, rb * cb), 256, 0, st>>>(B, rb, cb, ldb, tb == 'C', Br, Bi, Bs); ozg::note_launch(); }
+    ozg::launch_pdl(ozg::z3m_split_kernel, ozg::grid_for(c, ra * ca), 256, 0, st, A, ra, ca, lda, ta == 'C', Ar, Ai, As);
+    ozg::launch_pdl(ozg::z3m_split_kernel, ozg::grid_for(c, rb * cb), 256, 0, st, B, rb, cb, ldb, tb == 'C', Br, Bi, Bs);
     OZG_CUDA(cudaGetLastError());
   }
   const char rta = ta == 'N' ? 'N' : 'T', rtb = tb == 'N' ? 'N' : 'T';
@@ -172,8 +174,8 @@ extern "C" int ozg_zgemm3m(ozg_ctx* c, char transa, char transb, int64_t m, int6
   {
     PhaseScope ps(c, OZG_PHASE_SPLIT);
     const int beta_zero = (beta[0] == 0.0 && beta[1] == 0.0) ? 1 : 0;
-    { ozg::z3m_combine_kernel<<<ozg::grid_for(c, m * n), 256, 0, st>>>(P1, P2, P3, m, n, alpha[0], alpha[1], beta[0],
-                                                                       beta[1], beta_zero, C, ldc); ozg::note_launch(); }
+    ozg::launch_pdl(ozg::z3m_combine_kernel, ozg::grid_for(c, m * n), 256, 0, st, P1, P2, P3, m, n, alpha[0], alpha[1], beta[0],
+                                                                       beta[1], beta_zero, C, ldc);
     OZG_CUDA(cudaGetLastError());
   }
   if (nsamp > 0) {
