@@ -140,8 +140,8 @@ int emu_gemm(ozg_ctx* c, bool cplx, char ta, char tb, int64_t m, int64_t n, int6
       hb.hist = hist + 10;
       if (e == cudaSuccess) e = ozg::launch_stats_pair(ha, hb, st);
     } else {
-      e = autos ? ozg::launch_rowmax(sa, st) : ozg::launch_split(sa, st);
-      if (e == cudaSuccess) e = autos ? ozg::launch_rowmax(sb, st) : ozg::launch_split(sb, st);
+      e = ozg::launch_rowmax_both(sa, sb, st);
+      if (!autos && e == cudaSuccess) e = ozg::launch_digits_pair(sa, sb, st);
     }
     delete split_scope;
     OZG_CUDA(e);
@@ -160,8 +160,7 @@ int emu_gemm(ozg_ctx* c, bool cplx, char ta, char tb, int64_t m, int64_t n, int6
   }
   if (autos) {
     PhaseScope ps(c, OZG_PHASE_SPLIT);
-    OZG_CUDA(ozg::launch_digits(sa, st));
-    OZG_CUDA(ozg::launch_digits(sb, st));
+    OZG_CUDA(ozg::launch_digits_pair(sa, sb, st));
   }
 
   CUtensorMap tmA, tmB[2];
@@ -324,8 +323,7 @@ int emu_gemm(ozg_ctx* c, bool cplx, char ta, char tb, int64_t m, int64_t n, int6
     ca.plane_to = cb.plane_to = nullptr;
     ca.gate = cb.gate = s_dev + 1;
     ca.diff = cb.diff = 0;  // the re-run reads digit planes only
-    OZG_CUDA(ozg::launch_digits(ca, st));
-    OZG_CUDA(ozg::launch_digits(cb, st));
+    OZG_CUDA(ozg::launch_digits_pair(ca, cb, st));
     ozg::GemmArgs g2 = ga;
     g2.s = s_rep;
     g2.s_dev = nullptr;

@@ -47,9 +47,6 @@ __device__ __forceinline__ double ld_op(const double* X, int64_t ld, char t, int
   return p[0];
 }
 
-// One warp per (call, sample); the call's error goes to its own slot of err_out.
-__device__ void check_one(const CheckArgs& P, int sample, int lane, double* err_slot);
-
 __global__ void check_pre(CheckArgs P) {
   pdl_entry();
   if (P.gate != nullptr && *P.gate) return;
@@ -95,41 +92,51 @@ __device__ __forceinline__ dd dot2_reduce_warp(dot2 a) {
   return fast_two_sum(a.s, a.c);
 }
 
-__device__ __forceinline__ dd exact_dot_reduce_warp(i128 a, int unit) {
+__device__ __forceinline__ void i128_reduce_warp(i128& a) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     const i128 other = {__shfl_xor_sync(0xffffffffu, a.lo, o), __shfl_xor_sync(0xffffffffu, a.hi, o)};
     i128_add(a, other);
   }
-  return i128_to_dd(a, unit);
 }
 
-__device__ void check_one(const CheckArgs& P, int sample, int lane, double* err_slot) {
+// One sample of a call, its k split over the NW warps of a block (thread `lane` of 32 NW; NW = 1: over
+// a warp); the error goes to err_slot.  A single call has few samples, and one warp walking k has
+// too few loads in flight: 64 samples at k = 1900 took 55 us with a warp each and take 19 with eight (sixteen: 35).
+template <int NW>
+__device__ __forceinline__ void check_one(const CheckArgs& P, int sample, int lane, double* err_slot) {
+  constexpr int T = 32 * NW;
+  __shared__ dd part_re[NW], part_im[NW];
+  __shared__ i128 part_acc[NW];
+  __shared__ double part_abs[NW];
   int64_t i, j;
   sample_ij(P, sample, i, j);
   dd re = {0, 0}, im = {0, 0};
   double sabs = 0.0;
-  if (!P.cplx && P.ea != nullptr && P.fb != nullptr && P.k < (1ll << 26)) {
-    const int unit = P.ea[i] + P.fb[j] - 100;
-    i128 acc = {0ull, 0ll};
-    for (int64_t l = lane; l < P.k; l += 32) {
+  i128 acc = {0ull, 0ll};
+  int unit = 0;
+  const bool exact = !P.cplx && P.ea != nullptr && P.fb != nullptr && P.k < (1ll << 26);
+  if (exact) {
+    unit = P.ea[i] + P.fb[j] - 100;
+#pragma unroll 4
+    for (int64_t l = lane; l < P.k; l += T) {
       const double ar = (P.ta == 'N') ? P.A[i + l * P.lda] : P.A[l + i * P.lda];
       const double br = (P.tb == 'N') ? P.B[l + j * P.ldb] : P.B[j + l * P.ldb];
       add_exact_term(acc, __double_as_longlong(ar), __double_as_longlong(br), unit);
       sabs = fma(fabs(ar), fabs(br), sabs);
     }
-    re = exact_dot_reduce_warp(acc, unit);
+    i128_reduce_warp(acc);
   } else if (!P.cplx) {
-    dot2 acc = {0.0, 0.0};
-    for (int64_t l = lane; l < P.k; l += 32) {
+    dot2 d2 = {0.0, 0.0};
+    for (int64_t l = lane; l < P.k; l += T) {
       const double ar = (P.ta == 'N') ? P.A[i + l * P.lda] : P.A[l + i * P.lda];
       const double br = (P.tb == 'N') ? P.B[l + j * P.ldb] : P.B[j + l * P.ldb];
-      dot2_add(acc, ar, br);
+      dot2_add(d2, ar, br);
       sabs = fma(fabs(ar), fabs(br), sabs);
     }
-    re = dot2_reduce_warp(acc);
+    re = dot2_reduce_warp(d2);
   }
-  for (int64_t l = lane; P.cplx && l < P.k; l += 32) {
+  for (int64_t l = lane; P.cplx && l < P.k; l += T) {
     double ai = 0, bi = 0;
     const double ar = ld_op(P.A, P.lda, P.ta, i, l, P.cplx, &ai);
     const double br = ld_op(P.B, P.ldb, P.tb, l, j, P.cplx, &bi);
@@ -147,7 +154,35 @@ __device__ void check_one(const CheckArgs& P, int sample, int lane, double* err_
     }
     sabs += __shfl_xor_sync(0xffffffffu, sabs, o);
   }
+  if (NW > 1) {  // the warps' parts, combined by the first warp
+    const int w = lane >> 5;
+    if ((lane & 31) == 0) {
+      part_re[w] = re;
+      part_im[w] = im;
+      part_acc[w] = acc;
+      part_abs[w] = sabs;
+    }
+    __syncthreads();
+    if (w != 0) return;
+    const bool has = lane < NW;
+    sabs = has ? part_abs[lane & (NW - 1)] : 0.0;
+    acc = has ? part_acc[lane & (NW - 1)] : i128{0ull, 0ll};
+    re = has ? part_re[lane & (NW - 1)] : dd{0, 0};
+    im = has ? part_im[lane & (NW - 1)] : dd{0, 0};
+#pragma unroll
+    for (int o = NW / 2; o > 0; o >>= 1) {
+      if (exact) {
+        const i128 other = {__shfl_xor_sync(0xffffffffu, acc.lo, o), __shfl_xor_sync(0xffffffffu, acc.hi, o)};
+        i128_add(acc, other);
+      } else {
+        re = dd_add(re, dd_shfl_xor(re, o));
+        if (P.cplx) im = dd_add(im, dd_shfl_xor(im, o));
+      }
+      sabs += __shfl_xor_sync(0xffffffffu, sabs, o);
+    }
+  }
   if (lane != 0) return;
+  if (exact) re = i128_to_dd(acc, unit);
   const double cr_old = P.beta_zero ? 0.0 : P.cold[2 * sample], ci_old = P.beta_zero ? 0.0 : P.cold[2 * sample + 1];
   double err;
   if (!P.cplx) {
@@ -191,12 +226,11 @@ __device__ void check_one(const CheckArgs& P, int sample, int lane, double* err_
   atomicMax(reinterpret_cast<unsigned long long*>(err_slot), (unsigned long long)__double_as_longlong(err));
 }
 
-__global__ void check_post(CheckArgs P) {
+constexpr int kCheckWarps = 8;
+__global__ void __launch_bounds__(32 * kCheckWarps) check_post(CheckArgs P) {
   pdl_entry();
   if (P.gate != nullptr && *P.gate) return;
-  const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-  if (warp >= P.nsamp) return;
-  check_one(P, warp, lane, P.err_out);
+  check_one<kCheckWarps>(P, (int)blockIdx.x, (int)threadIdx.x, P.err_out);
 }
 
 // batched: calls[c] with nsamp samples each; warp w -> call w / nsamp, sample w % nsamp
@@ -223,7 +257,7 @@ __global__ void check_post_batched(const CheckArgs* calls, int ncalls, int nsamp
   const int* gate = Pp->gate;  // read the gate before anything else (most re-run checks skip)
   if (gate != nullptr && *gate) return;
   const CheckArgs P = *Pp;
-  check_one(P, (int)(warp % nsamp), lane, P.err_out);
+  check_one<1>(P, (int)(warp % nsamp), lane, P.err_out);
 }
 
 }  // namespace
@@ -258,8 +292,7 @@ cudaError_t launch_check_post(const CheckArgs& a, cudaStream_t st) {
   cudaError_t e = cudaMemsetAsync(a.err_out, 0, sizeof(double), st);
   if (e == cudaSuccess && a.part_err != nullptr) e = cudaMemsetAsync(a.part_err, 0, 2 * sizeof(double), st);
   if (e != cudaSuccess) return e;
-  const int warps_per_block = 4;
-  launch_pdl(check_post, (a.nsamp + warps_per_block - 1) / warps_per_block, 32 * warps_per_block, 0, st, a);
+  launch_pdl(check_post, a.nsamp, 32 * kCheckWarps, 0, st, a);
   return cudaGetLastError();
 }
 

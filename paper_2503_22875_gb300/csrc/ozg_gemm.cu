@@ -1146,15 +1146,16 @@ __global__ void __launch_bounds__(THREADS, 1)
   if (P.kd != 0 && P.s_dev != nullptr && *P.s_dev <= P.kd) return;
   stacked_body<false, true>(&tmA, &tmB, &P, nullptr);
 }
-// Rounds the window sums of the split kernel and writes C: a block per tile and chunk of 8 outputs,
-// a thread per row.  HBM / L2 bound: 8 bytes read per output and window.
+// Rounds the window sums of the split kernel and writes C: a block per tile and chunk of kFin
+// outputs, a thread per row.  L2 bound: 8 bytes read per output and window.
+constexpr int kFin = 4;
 __global__ void __launch_bounds__(BM) split_finish_kernel(const GemmArgs P) {
   pdl_entry();
   if (P.nonfinite != nullptr && *P.nonfinite) return;
   if (P.kd != 0 && P.s_dev != nullptr && *P.s_dev <= P.kd) return;
-  const int chunks = P.cplx ? 8 : 16;
+  const int chunks = (P.cplx ? 64 : 128) / kFin;
   TileJob j = get_job<128, 2, false>((int)(blockIdx.x / chunks), nullptr, nullptr, &P, nullptr);
-  const int o = (int)(blockIdx.x % chunks) * 8, r = threadIdx.x;
+  const int o = (int)(blockIdx.x % chunks) * kFin, r = threadIdx.x;
   const int win = window_len(j.s, (int64_t)j.KB * 128, j.cplx);
   const int64_t grow = (int64_t)j.tm * BM + r;
   PushArgs pa;
@@ -1169,10 +1170,10 @@ __global__ void __launch_bounds__(BM) split_finish_kernel(const GemmArgs P) {
       reinterpret_cast<const long long*>(P.Wsplit) + (size_t)(blockIdx.x / chunks) * P.part_windows * BM * 128 + (size_t)o * BM + r;
   const int64_t c0 = (j.cplx ? (pa.gcol0 >> 1) : pa.gcol0) + o, climit = j.cplx ? j.n : j.cols;
   if (c0 >= climit) return;
-  long long s0[8], rw[8];
-  int fe[8];
+  long long s0[kFin], rw[kFin];
+  int fe[kFin];
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
+  for (int i = 0; i < kFin; ++i) {
     rw[i] = __ldcg(Wt + (size_t)i * BM);
     fe[i] = c0 + i < climit ? __ldg(j.f + c0 + i) : 0;
     s0[i] = 0;
@@ -1180,7 +1181,7 @@ __global__ void __launch_bounds__(BM) split_finish_kernel(const GemmArgs P) {
   int widx = 0, wstart = 2, wlen = stk_len0(j.s, win);
   for (; wstart + wlen <= j.s + 1; ++widx) {  // the last window's words end in rw, the earlier ones' in s0
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
+    for (int i = 0; i < kFin; ++i) {
       s0[i] = widx == 0 ? rw[i] : close_val(s0[i], rw[i], widx, wlen);
       rw[i] = __ldcg(Wt + (size_t)(widx + 1) * BM * 128 + (size_t)i * BM);
     }
@@ -1189,7 +1190,7 @@ __global__ void __launch_bounds__(BM) split_finish_kernel(const GemmArgs P) {
   }
   pa.widx = widx;
   pa.wlen = wlen;
-  window_out<8, false, true>(rw, o, pa, j, s0, fe);
+  window_out<kFin, false, true>(rw, o, pa, j, s0, fe);
 }
 __global__ void __launch_bounds__(THREADS, 1) slice_gemm_grouped_stacked_kernel(const GroupArgs G) {
   if (G.run != nullptr && *G.run == 0) return;
@@ -1363,7 +1364,7 @@ cudaError_t launch_slice_gemm(const CUtensorMap& tmA, const CUtensorMap& tmB, co
       return cudaErrorInvalidValue;
     launch_pdl(slice_gemm_split_kernel, a.grid, THREADS, stk::SMEM, st, tmA, tmB, a);
     const int64_t tiles = ((a.rows + BM - 1) / BM) * ((a.cols + 127) / 128);
-    launch_pdl(split_finish_kernel, (unsigned)(tiles * (a.cplx ? 8 : 16)), BM, 0, st, a);
+    launch_pdl(split_finish_kernel, (unsigned)(tiles * ((a.cplx ? 64 : 128) / kFin)), BM, 0, st, a);
     return cudaGetLastError();
   }
   // a plane set with differences is read by the stacked kernel only

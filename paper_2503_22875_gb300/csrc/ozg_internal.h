@@ -75,6 +75,9 @@ cudaError_t launch_split(const SplitArgs& a, cudaStream_t st);
 // the two passes of launch_split (row maxima; digits over the plane range of a)
 cudaError_t launch_rowmax(const SplitArgs& a, cudaStream_t st);
 cudaError_t launch_digits(const SplitArgs& a, cudaStream_t st);
+// the same for both operands of a call (same type, k and plane layout; maxbits zeroed)
+cudaError_t launch_rowmax_both(const SplitArgs& a, const SplitArgs& b, cudaStream_t st);
+cudaError_t launch_digits_pair(const SplitArgs& a, const SplitArgs& b, cudaStream_t st);
 
 // int8 copy of fp16 digit planes (inspection path): out[p][r][l] = D[p][r][l], l < k
 cudaError_t launch_digits_to_i8(const __half* D, int64_t planes, int64_t plane_rows, int64_t k, int64_t Kp,

@@ -123,17 +123,83 @@ __global__ void rowmax_strided(const double* __restrict__ X, int64_t ld, int64_t
   }
 }
 
+// ---------------------------------------------------------------- row maxima, both operands of a small call
+// One launch whose blocks have eight loads in flight per thread: 32 rows x 64 k of a strided operand
+// (lanes along the rows, the eight warps along k), 8 rows x 256 k of a contiguous one (a warp per
+// row).  Latency bound: a launch per operand with one load in flight per thread took 4.1 + 3.7 us at
+// 256 x 256, 9.1 + 9.1 at 768 x 768 complex.  Partial maxima merge by atomicMax.
+constexpr int kRpLoads = 8, kRpStridedK = 8 * kRpLoads, kRpContigK = 32 * kRpLoads;
+template <int CPLX>
+__device__ __forceinline__ uint64_t abs_elem(const double* X, int64_t idx) {
+  if (!CPLX) return __ldg(reinterpret_cast<const uint64_t*>(X) + idx) & kAbsMask;
+  const ulonglong2 v = __ldg(reinterpret_cast<const ulonglong2*>(X) + idx);
+  const uint64_t a = v.x & kAbsMask, b = v.y & kAbsMask;
+  return a > b ? a : b;
+}
+template <int CPLX>
+__global__ void __launch_bounds__(256) rowmax_pair(const SplitArgs a, const SplitArgs b, unsigned blocks_a) {
+  pdl_entry();
+  __shared__ unsigned long long red[8][32];
+  const bool first = blockIdx.x < blocks_a;
+  const SplitArgs& J = first ? a : b;
+  const unsigned block = first ? blockIdx.x : blockIdx.x - blocks_a;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int64_t rows = J.rows, k = J.k, ld = J.ld;
+  uint64_t v[kRpLoads], mx = 0;
+  if (J.strided) {
+    const unsigned kt = (unsigned)((k + kRpStridedK - 1) / kRpStridedK);
+    const int64_t row = (int64_t)(block / kt) * 32 + lane, l0 = (int64_t)(block % kt) * kRpStridedK + w;
+#pragma unroll
+    for (int i = 0; i < kRpLoads; ++i) {
+      const int64_t l = l0 + 8 * i;
+      v[i] = row < rows && l < k ? abs_elem<CPLX>(J.X, row + l * ld) : 0ull;
+    }
+#pragma unroll
+    for (int i = 0; i < kRpLoads; ++i) mx = v[i] > mx ? v[i] : mx;
+    red[w][lane] = mx;
+    __syncthreads();
+    if (w != 0) return;
+#pragma unroll
+    for (int i = 1; i < 8; ++i) mx = red[i][lane] > mx ? red[i][lane] : mx;
+    if (row < rows && mx) {
+      atomicMax(&J.maxbits[row], mx);
+      flag_nonfinite(mx, J.nonfinite);
+    }
+  } else {
+    const unsigned kt = (unsigned)((k + kRpContigK - 1) / kRpContigK);
+    const int64_t row = (int64_t)(block / kt) * 8 + w, l0 = (int64_t)(block % kt) * kRpContigK + lane;
+    if (row >= rows) return;
+#pragma unroll
+    for (int i = 0; i < kRpLoads; ++i) {
+      const int64_t l = l0 + 32 * i;
+      v[i] = l < k ? abs_elem<CPLX>(J.X, l + row * ld) : 0ull;
+    }
+#pragma unroll
+    for (int i = 0; i < kRpLoads; ++i) mx = v[i] > mx ? v[i] : mx;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const uint64_t t = __shfl_xor_sync(0xffffffffu, mx, o);
+      mx = t > mx ? t : mx;
+    }
+    if (lane == 0 && mx) {
+      atomicMax(&J.maxbits[row], (unsigned long long)mx);
+      flag_nonfinite(mx, J.nonfinite);
+    }
+  }
+}
+
 // ---------------------------------------------------------------- digits, contiguous rows
 // thread per (row, group of 8 consecutive l); 16-byte stores per digit plane
 template <int CPLX, int KD>
-__global__ void digits_contig(const double* __restrict__ X, int64_t ld, int64_t rows, int64_t k, int conj, int s,
-                              int64_t Kp, int64_t plane_rows, const unsigned long long* __restrict__ maxbits,
-                              int32_t* __restrict__ exps, __half* __restrict__ D, PlaneRange pr) {
-  pdl_entry();
-  int t_lo, t_hi;
-  if (!pr.resolve(s, t_lo, t_hi)) return;
+__device__ __forceinline__ void digits_contig(const SplitArgs& J, const PlaneRange& pr, int t_lo, int t_hi, unsigned block) {
+  const double* X = J.X;
+  const int64_t ld = J.ld, rows = J.rows, k = J.k, Kp = J.Kp, plane_rows = J.plane_rows;
+  const int conj = J.conj;
+  const unsigned long long* maxbits = J.maxbits;
+  int32_t* exps = J.exps;
+  __half* D = J.D;
   int64_t groups = (k + 7) / 8;
-  int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  int64_t gid = (int64_t)block * 256 + threadIdx.x;
   if (gid >= rows * groups) return;
   int64_t row = gid / groups, l0 = (gid % groups) * 8;
   int e = exponent_from_maxbits(maxbits[row]);
@@ -161,18 +227,18 @@ __global__ void digits_contig(const double* __restrict__ X, int64_t ld, int64_t 
 // ---------------------------------------------------------------- digits, strided rows
 // block: 32 rows x 64 l tile staged (transposed) through shared memory
 template <int CPLX, int KD>
-__global__ void __launch_bounds__(256) digits_strided(const double* __restrict__ X, int64_t ld, int64_t rows,
-                                                      int64_t k, int conj, int s, int64_t Kp, int64_t plane_rows,
-                                                      const unsigned long long* __restrict__ maxbits,
-                                                      int32_t* __restrict__ exps, __half* __restrict__ D,
-                                                      PlaneRange pr) {
-  pdl_entry();
-  int t_lo, t_hi;
-  if (!pr.resolve(s, t_lo, t_hi)) return;
+__device__ __forceinline__ void digits_strided(const SplitArgs& J, const PlaneRange& pr, int t_lo, int t_hi, unsigned block) {
+  const double* X = J.X;
+  const int64_t ld = J.ld, rows = J.rows, k = J.k, Kp = J.Kp, plane_rows = J.plane_rows;
+  const int conj = J.conj;
+  const unsigned long long* maxbits = J.maxbits;
+  int32_t* exps = J.exps;
+  __half* D = J.D;
   constexpr int TR = 32, TL = 64;
   constexpr int W = CPLX ? 2 : 1;
   __shared__ uint64_t tile[TL][TR * W + 1];
-  int64_t r0 = (int64_t)blockIdx.x * TR, l0 = (int64_t)blockIdx.y * TL;
+  const unsigned row_blocks = (unsigned)((rows + TR - 1) / TR);
+  int64_t r0 = (int64_t)(block % row_blocks) * TR, l0 = (int64_t)(block / row_blocks) * TL;
   int tid = threadIdx.x;
   // load: thread -> (row = tid % 32, l = tid / 32 + 8 j)
   {
@@ -207,6 +273,24 @@ __global__ void __launch_bounds__(256) digits_strided(const double* __restrict__
     int64_t orow = CPLX ? 2 * row + part : row;
     store_planes8<KD>(b, e, t_lo, t_hi, D + orow * Kp + l0 + lg, plane_rows * Kp, pr);
   }
+}
+
+// The digits of one or both operands of a call: blocks 0 .. blocks_a - 1 work on a, the others on b.
+// ROWS: the rows' layout, 0 contiguous, 1 strided, 2 either (one launch for operands of both kinds,
+// which carries the registers and shared memory of the larger path).
+template <int CPLX, int KD, int ROWS>
+__global__ void __launch_bounds__(256) digits_kernel(const SplitArgs a, const SplitArgs b, unsigned blocks_a) {
+  pdl_entry();
+  const bool first = blockIdx.x < blocks_a;
+  const SplitArgs& J = first ? a : b;
+  const PlaneRange pr{J.plane_from, J.plane_to, J.gate, J.kd, J.diff};
+  int t_lo, t_hi;
+  if (!pr.resolve(J.s, t_lo, t_hi)) return;
+  const unsigned block = first ? blockIdx.x : blockIdx.x - blocks_a;
+  if (ROWS == 1 || (ROWS == 2 && J.strided))
+    digits_strided<CPLX, KD>(J, pr, t_lo, t_hi, block);
+  else
+    digits_contig<CPLX, KD>(J, pr, t_lo, t_hi, block);
 }
 
 __global__ void digits_to_i8(const __half* __restrict__ D, int64_t planes_rows, int64_t k, int64_t Kp,
@@ -246,38 +330,67 @@ cudaError_t launch_rowmax(const SplitArgs& a, cudaStream_t st) {
 }
 
 namespace {
-template <int CPLX, int KD>
-void digits_launch(const SplitArgs& a, cudaStream_t st) {
-  const PlaneRange pr{a.plane_from, a.plane_to, a.gate, a.kd, a.diff};
-  const int64_t kk = a.k > 0 ? a.k : 1;
-  if (!a.strided || a.k == 0) {
-    const int64_t total = a.rows * ((kk + 7) / 8);
-    launch_pdl(digits_contig<CPLX, KD>, (unsigned)((total + 255) / 256), 256, 0, st, 
-        a.X, a.ld, a.rows, a.k, a.conj, a.s, a.Kp, a.plane_rows, a.maxbits, a.exps, a.D, pr);
-  } else {
-    const dim3 grid((unsigned)((a.rows + 31) / 32), (unsigned)((a.k + 63) / 64));
-    launch_pdl(digits_strided<CPLX, KD>, grid, 256, 0, st, a.X, a.ld, a.rows, a.k, a.conj, a.s, a.Kp, a.plane_rows, a.maxbits,
-                                                   a.exps, a.D, pr);
-  }
+unsigned digit_blocks(const SplitArgs& a) {
+  if (a.rows <= 0 || a.k <= 0) return 0;
+  return (unsigned)(a.strided ? ((a.rows + 31) / 32) * ((a.k + 63) / 64) : (a.rows * ((a.k + 7) / 8) + 255) / 256);
 }
+template <int CPLX, int KD>
+void digits_launch_as(const SplitArgs& a, const SplitArgs& b, unsigned blocks_a, unsigned blocks, cudaStream_t st) {
+  if (a.strided != b.strided)
+    launch_pdl(digits_kernel<CPLX, KD, 2>, blocks, 256, 0, st, a, b, blocks_a);
+  else if (a.strided)
+    launch_pdl(digits_kernel<CPLX, KD, 1>, blocks, 256, 0, st, a, b, blocks_a);
+  else
+    launch_pdl(digits_kernel<CPLX, KD, 0>, blocks, 256, 0, st, a, b, blocks_a);
+}
+cudaError_t digits_launch(const SplitArgs& a, const SplitArgs& b, unsigned blocks_a, unsigned blocks, cudaStream_t st) {
+  if (blocks == 0) return cudaSuccess;
+  if (a.cplx) {
+    if (a.kd) digits_launch_as<1, 1>(a, b, blocks_a, blocks, st);
+    else digits_launch_as<1, 0>(a, b, blocks_a, blocks, st);
+  } else {
+    if (a.kd) digits_launch_as<0, 1>(a, b, blocks_a, blocks, st);
+    else digits_launch_as<0, 0>(a, b, blocks_a, blocks, st);
+  }
+  return cudaGetLastError();
+}
+// elements (real numbers) of both operands up to which a launch covers both at some cost per element
+constexpr int64_t kPairElems = 4 << 20;
+bool small_pair(const SplitArgs& a, const SplitArgs& b) { return (a.rows + b.rows) * a.k * (a.cplx ? 2 : 1) <= kPairElems; }
 }  // namespace
 
 cudaError_t launch_digits(const SplitArgs& a, cudaStream_t st) {
-  if (a.rows <= 0) return cudaSuccess;
-  if (a.cplx) {
-    if (a.kd) digits_launch<1, 1>(a, st);
-    else digits_launch<1, 0>(a, st);
-  } else {
-    if (a.kd) digits_launch<0, 1>(a, st);
-    else digits_launch<0, 0>(a, st);
-  }
-  return cudaGetLastError();
+  return digits_launch(a, a, digit_blocks(a), digit_blocks(a), st);
+}
+cudaError_t launch_digits_pair(const SplitArgs& a, const SplitArgs& b, cudaStream_t st) {
+  if (a.strided == b.strided || small_pair(a, b))
+    return digits_launch(a, b, digit_blocks(a), digit_blocks(a) + digit_blocks(b), st);
+  cudaError_t e = launch_digits(a, st);
+  return e == cudaSuccess ? launch_digits(b, st) : e;
 }
 
 cudaError_t launch_split(const SplitArgs& a, cudaStream_t st) {
   cudaError_t e = launch_rowmax(a, st);
   if (e != cudaSuccess) return e;
   return launch_digits(a, st);
+}
+
+// Row maxima of both operands (maxbits zeroed): one launch for small ones; large ones, which fill the
+// GPU by themselves, a streaming launch each.
+cudaError_t launch_rowmax_both(const SplitArgs& a, const SplitArgs& b, cudaStream_t st) {
+  if (small_pair(a, b)) {
+    auto blocks = [](const SplitArgs& x) {
+      return (unsigned)(x.strided ? ((x.rows + 31) / 32) * ((x.k + kRpStridedK - 1) / kRpStridedK)
+                                  : ((x.rows + 7) / 8) * ((x.k + kRpContigK - 1) / kRpContigK));
+    };
+    const unsigned ba = blocks(a), bb = blocks(b);
+    if (ba + bb == 0) return cudaSuccess;
+    if (a.cplx) launch_pdl(rowmax_pair<1>, ba + bb, 256, 0, st, a, b, ba);
+    else launch_pdl(rowmax_pair<0>, ba + bb, 256, 0, st, a, b, ba);
+    return cudaGetLastError();
+  }
+  cudaError_t e = launch_rowmax(a, st);
+  return e == cudaSuccess ? launch_rowmax(b, st) : e;
 }
 
 cudaError_t launch_digits_to_i8(const __half* D, int64_t planes, int64_t plane_rows, int64_t k, int64_t Kp,

