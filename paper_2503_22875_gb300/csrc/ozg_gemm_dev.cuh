@@ -387,13 +387,18 @@ __device__ __forceinline__ void window_out(const long long* rw, int o0, const Pu
       continue;
     }
     if (!j.cplx) {
+      // the bound and the pointer in few instructions: 64-bit products per output cost 2%
+      // (6000 x 6000 x 192 644 -> 629 us)
+      const int left = a.row_ok ? (int)min((int64_t)RB, j.cols - (c0 + i0)) : 0;
+      double* cp = j.C + a.orow + (c0 + i0) * j.ldc;
+      if (a.unit_ab) {
 #pragma unroll
-      for (int i = 0; i < RB; ++i) {
-        const int64_t col = c0 + i0 + i;
-        if (a.row_ok && col < j.cols) {
-          double* cp = j.C + a.orow + col * j.ldc;
-          __stcs(cp, a.unit_ab ? tv[i] : (j.beta_zero ? j.a0 * tv[i] : fma(j.a0, tv[i], j.b0 * *cp)));
-        }
+        for (int i = 0; i < RB; ++i, cp += j.ldc)
+          if (i < left) __stcs(cp, tv[i]);
+      } else {
+#pragma unroll
+        for (int i = 0; i < RB; ++i, cp += j.ldc)
+          if (i < left) __stcs(cp, j.beta_zero ? j.a0 * tv[i] : fma(j.a0, tv[i], j.b0 * *cp));
       }
     } else {
 #pragma unroll
