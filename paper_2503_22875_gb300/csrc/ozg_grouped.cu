@@ -47,8 +47,16 @@ void destroy_plan(GroupPlan* p) {
 
 namespace {
 
-uint64_t fnv(uint64_t h, const void* p, size_t n) {
+// Hash of a batch's description, eight bytes a step (a byte a step took 35 us for 256 calls).  The
+// shift brings high bits down again: a multiplication alone would let two flipped sign bits cancel.
+uint64_t batch_hash(uint64_t h, const void* p, size_t n) {
   const unsigned char* b = static_cast<const unsigned char*>(p);
+  for (; n >= 8; n -= 8, b += 8) {
+    uint64_t w;
+    std::memcpy(&w, b, 8);
+    h = (h ^ w) * 0x9E3779B97F4A7C15ull;
+    h ^= h >> 32;
+  }
   for (size_t i = 0; i < n; ++i) h = (h ^ b[i]) * 1099511628211ull;
   return h;
 }
@@ -625,11 +633,11 @@ int grouped_call(ozg_ctx* c, int64_t count, const ozg_gemm_desc* descs, const in
     wauto[i] = autom_all[widx[i]];
   }
   uint64_t key = 1469598103934665603ull;
-  key = fnv(key, work.data(), sizeof(ozg_gemm_desc) * n);
-  key = fnv(key, ws.data(), sizeof(int) * n);
-  key = fnv(key, &c->check_samples, sizeof(int));
-  key = fnv(key, &c->autotune, sizeof(int));
-  key = fnv(key, wauto.data(), n);
+  key = batch_hash(key, work.data(), sizeof(ozg_gemm_desc) * n);
+  key = batch_hash(key, ws.data(), sizeof(int) * n);
+  key = batch_hash(key, &c->check_samples, sizeof(int));
+  key = batch_hash(key, &c->autotune, sizeof(int));
+  key = batch_hash(key, wauto.data(), n);
 
   GroupPlan* P = c->plan.get();
   const bool reuse = P && P->key == key && P->epoch == c->gws_epoch;
