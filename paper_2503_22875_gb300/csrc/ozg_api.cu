@@ -1,7 +1,8 @@
 // C ABI (include/ozg.h): argument checking with BLAS xerbla numbering, quick returns,
 // workspace management and the launch sequence of the emulated GEMM:
-//   split(op(A)) -> split(op(B)) -> fused slice-GEMM + epilogue -> native kernel gated on
-//   the non-finite flag (runs only if an input held Inf/NaN).
+//   split(op(A), op(B)) -> slice products with the epilogue (on difference planes, on tiles, or on
+//   parts of tiles and a finishing kernel) -> native kernel gated on the non-finite flag (runs only
+//   if an input held Inf/NaN).
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
@@ -48,7 +49,7 @@ int emu_gemm(ozg_ctx* c, bool cplx, char ta, char tb, int64_t m, int64_t n, int6
   if (autos) s = std::max(c->sel_s_hi, s_fb);
   const int nsamp = autos ? std::max(c->check_samples, 64) : c->check_samples;
   const bool beta_zero0 = (beta[0] == 0.0 && (!cplx || beta[1] == 0.0));
-  const int64_t Kp = ozg::plane_pitch(k);
+  int64_t Kp = ozg::plane_pitch(k, false);
   const int64_t prA = cplx ? 2 * m : m, prB = cplx ? 2 * n : n;
   const int BM = ozg::slice_gemm_tile_m();
   auto grid_of = [&](int variant) {
@@ -87,6 +88,10 @@ int emu_gemm(ozg_ctx* c, bool cplx, char ta, char tb, int64_t m, int64_t n, int6
   layout();
   if ((kd || plan.parts > 1) && !ws_available(c, cv.off)) {  // without either where the memory is not there
     plan = SinglePlan();
+    layout();
+  }
+  if (!ws_available(c, cv.off)) {  // nor for planes on whole 128-byte lines
+    Kp = ozg::plane_pitch(k, true);
     layout();
   }
   int rc = ensure_ws(c, cv.off);

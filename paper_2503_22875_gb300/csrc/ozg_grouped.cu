@@ -188,7 +188,7 @@ int check_desc(const ozg_gemm_desc& d, char& ta, char& tb) {
 // Build (upload) the plan's tables for `variant` into the grouped workspace.
 int build_plan(ozg_ctx* c, int64_t count, const ozg_gemm_desc* d, const std::vector<int>& s,
                const std::vector<char>& TA, const std::vector<char>& TB, const std::vector<char>& autom, int variant,
-               GroupPlan* P) {
+               GroupPlan* P, bool tight = false) {
   // s[i]: slice count of fixed calls; for automatic calls the fallback count (a cost estimate
   // and the re-run count), while their digit planes are written for the selector's top class
   int any_auto = 0;
@@ -226,7 +226,7 @@ int build_plan(ozg_ctx* c, int64_t count, const ozg_gemm_desc* d, const std::vec
   P->oMax = max0;
   P->max_bytes = cv.off - max0;
   for (int64_t i = 0; i < count; ++i) {
-    const int64_t Kp = plane_pitch(d[i].k);
+    const int64_t Kp = plane_pitch(d[i].k, tight);
     oEA[i] = cv.take(4 * (size_t)d[i].m);
     oEB[i] = cv.take(4 * (size_t)d[i].n);
     oDA[i] = cv.take((size_t)planes[i] * d[i].m * Kp * 2);
@@ -300,6 +300,7 @@ int build_plan(ozg_ctx* c, int64_t count, const ozg_gemm_desc* d, const std::vec
     }
     P->save_units = sp[count];
   }
+  if (!tight && !gws_available(c, cv.off)) return build_plan(c, count, d, s, TA, TB, autom, variant, P, true);
   int rc = ensure_gws(c, cv.off);
   if (rc) return rc;
   P->epoch = c->gws_epoch;
@@ -311,7 +312,7 @@ int build_plan(ozg_ctx* c, int64_t count, const ozg_gemm_desc* d, const std::vec
   std::vector<CheckArgs> chk(count);
   int* flags = gat<int>(c, P->oFlags);
   for (int64_t i = 0; i < count; ++i) {
-    const int64_t Kp = plane_pitch(d[i].k);
+    const int64_t Kp = plane_pitch(d[i].k, tight);
     SplitArgs a;
     a.X = d[i].A;
     a.ld = d[i].lda;

@@ -61,8 +61,8 @@ static int grow_buffer(ozg_ctx* c, void** buf, size_t* cap, size_t bytes) {
   return OZG_OK;
 }
 
-bool ws_available(ozg_ctx* c, size_t bytes) {
-  if (bytes <= c->ws_cap) return true;
+static bool room_for(ozg_ctx* c, size_t cap, size_t bytes) {
+  if (bytes <= cap) return true;
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(c->stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
     cudaGetLastError();
@@ -73,8 +73,11 @@ bool ws_available(ozg_ctx* c, size_t bytes) {
     cudaGetLastError();
     return false;
   }
-  return bytes + bytes / 8 + ((size_t)64 << 20) <= free_b + c->ws_cap;
+  return bytes + bytes / 8 + ((size_t)64 << 20) <= free_b + cap;
 }
+
+bool ws_available(ozg_ctx* c, size_t bytes) { return room_for(c, c->ws_cap, bytes); }
+bool gws_available(ozg_ctx* c, size_t bytes) { return room_for(c, c->gws_cap, bytes); }
 
 int ensure_ws(ozg_ctx* c, size_t bytes) { return grow_buffer(c, &c->ws, &c->ws_cap, bytes); }
 int ensure_z3ws(ozg_ctx* c, size_t bytes) { return grow_buffer(c, &c->z3ws, &c->z3ws_cap, bytes); }

@@ -7,8 +7,9 @@ namespace ozg {
 // Row pitch of a digit plane in elements (fp16): whole 128-byte lines, so that the 128-byte row of a
 // TMA box is one line.  With rows only 16-byte aligned every box row straddles two: 1537 x
 // 2001 with k = 1111, s = 10 took 639 us instead of 540, the learned batch of 2048 uneven calls 28.4
-// ms instead of 27.4.
-__host__ __device__ inline int64_t plane_pitch(int64_t k) { return (k + 63) / 64 * 64; }
+// ms instead of 27.4.  tight: 16-byte rows, for calls whose workspace does not have the room (a short
+// k's planes take up to eight times the space on whole lines).
+inline int64_t plane_pitch(int64_t k, bool tight) { return tight ? (k + 7) / 8 * 8 : (k + 63) / 64 * 64; }
 
 // Difference planes.  For up to kd slices a plane set holds, in blocks t = 1 .. kd, the digit plane
 // t and then the planes of digit p minus digit q for p < q, p + q = t + 1 (p = 1, 2, ..): the
