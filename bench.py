@@ -598,9 +598,13 @@ def single_section(ozg, torch, size, steps, phis=SINGLE_PHIS, slice_list=tuple(r
             ph = ctx.phase_times()
             ctx.set_profiling(False)
             gemm_ms = ph["gemm"][0] / max(ph["gemm"][1], 1)
-            # single calls of at most 16 slices run the stacked group-pair kernel (variant 5)
-            kname = "slice_gemm_stacked_kernel" if s <= 16 else "slice_gemm_kernel"
-            roof = tensor_roofline(kname, s * (s + 1) / 2 * flops, gemm_ms, f"slice_gemm_{n}_s{s}", 5 if s <= 16 else None)
+            # large single calls of at most 12 slices run on difference planes (s + s^2 / 4 products), others
+            # of at most 16 the stacked group pairs (variant 5: the triangle's products)
+            diff = n >= 4096 and s <= 12
+            kname = "slice_gemm_kd_kernel" if diff else "slice_gemm_stacked_kernel" if s <= 16 else "slice_gemm_kernel"
+            products = s + s * s // 4 if diff else s * (s + 1) // 2
+            roof = tensor_roofline(kname, products * flops, gemm_ms, f"slice_gemm_{n}_s{s}",
+                                   5 if s <= 16 and not diff else None)
             roof["slices"] = s
             roof["algorithmic_bytes"] = 2.0 * s * 2 * n * n + 8.0 * n * n
             ms_nat = timed(torch, st, lambda: ctx.native_dgemm("N", "N", n, n, n, 1.0, dA, n, dB, n, 0.0, dC, n), 1,

@@ -275,7 +275,8 @@ int ozg_set_fallback_slices(ozg_ctx* ctx, int slices);
  * pair), up to 16 slices; a call with more slices, the exact epilogue or the group-product
  * export runs as variant 1.  All variants give bit-identical C while the exact sum needs at most
  * two int64 windows (s <= 10 at any k); beyond that the FP64 continuation may round differently
- * in the last bits between the 256- and 128-wide families. */
+ * in the last bits between the 256- and 128-wide families.  A forced variant runs as named, without
+ * difference planes or cuts along k. */
 #define OZG_NUM_TILE_VARIANTS 6
 
 /* Tile-variant autotuner: enable != 0 times the variants the first time a shape bucket
@@ -283,8 +284,11 @@ int ozg_set_fallback_slices(ozg_ctx* ctx, int slices);
  * variant) is seen, keeps the fastest,
  * and appends single-call choices to cache_path (may be NULL) as "bucket variant" lines that
  * later contexts read back.  Tuning runs only for calls with beta == 0 (C is then write-only);
- * other calls use the heuristic: the stacked group pairs (variant 5) for single calls with at
- * most 16 slices outside the exact epilogue; otherwise the width that pads least, then for
+ * other calls use the heuristic: single calls with at most 16 slices outside the exact epilogue
+ * run on difference planes (A_p B_q + A_q B_p from three products of which two are shared: s + s^2 / 4
+ * products instead of s (s + 1) / 2), or on the stacked group pairs (variant 5), there with few
+ * tiles cut along k, whichever a cost model expects to be fastest (the tuner and its saved choices
+ * apply to calls that the model leaves on the tile variants); otherwise the width that pads least, then for
  * 128 x 256 tiles deferral when k >= 2048 (for a grouped batch, the mean k weighted by m n s^2)
  * and for 128 x 128 tiles variant 5 in grouped calls whose slice counts allow it, else two k
  * slices per stage (variant 1). */
