@@ -331,6 +331,17 @@ int ozg_debug_group_products(ozg_ctx* ctx, char transa, char transb, int64_t m, 
                              const double* A, int64_t lda, const double* B, int64_t ldb, int slices,
                              int64_t* G_out);
 
+/* How a single call is planned on a device of num_sms SMs, when no tile variant is forced, the exact
+ * epilogue is off and the workspace has the room (computed on the host; needs no context or GPU).
+ * slices: 1..18, or 0: a learned call with the selector's largest class sel_max and the fallback count
+ * (both ignored otherwise).  plan[4] receives
+ *   [0] the largest slice count that runs on difference planes (0: none),
+ *   [1] the parts every tile's k range is cut into (1: whole tiles; 1 with difference planes),
+ *   [2] 64-wide k sub-tiles per part, [3] window words per output a cut call keeps.
+ * Returns 0 or OZG_ERR_INVALID. */
+int ozg_debug_single_plan(int num_sms, int cplx, int64_t m, int64_t n, int64_t k, int slices, int sel_max,
+                          int fallback, int* plan);
+
 /* ---- fault-path hooks (tests; no GPU fault is involved) ----
  * ozg_debug_wait: queues one CTA that waits on an mbarrier nothing arrives at, bounded at
  * `cycles` clock cycles (1000 .. 4e9); when the wait runs out, the kernel raises the

@@ -600,6 +600,7 @@ constexpr int NOUT = 64;                     // outputs per epilogue thread (rea
 constexpr uint32_t DSLOT = SLOT >> 4;         // descriptor start-address units per ring entry
 static_assert(SMEM <= 227 * 1024, "stage ring");
 static_assert(SMEM < (1u << 18), "descriptor start addresses stay within their 14-bit field");
+static_assert(Cfg<128, 2>::SK == kStackedK, "the padded k of stk_kpad");
 }  // namespace stk
 
 // The four K = 16 MMAs of one 64-wide k sub-tile; the first overwrites the accumulator when it
@@ -620,16 +621,6 @@ __device__ __forceinline__ void stk_pass(int wstart, int wlen, int q, int& ga, b
     two = true;
     ga = wstart + 2 * q;
   }
-}
-// Length of the first window.  With three or more windows every window but the last holds win
-// groups, as in the one-group kernels (their FP64 continuation rounds per window, so the split
-// must be the same for the same bits).  With two windows the exact sum is rounded once and any
-// split into windows of at most win groups gives the same bits: the first takes one group
-// less when that makes the second window's count even (a lone group of a later window pairs
-// far more planes than the lone group 2 of the first).
-__device__ __forceinline__ int stk_len0(int s, int win) {
-  if (s <= win || s > 2 * win) return min(s, win);
-  return (((win - s) & 1) && s - (win - 1) <= win) ? win - 1 : win;
 }
 // k sweeps per chain: a sweep adds ga (two groups) or ga - 1 (lone group) 64-k MMA stages to
 // the accumulator columns that collect the most
@@ -718,7 +709,7 @@ __device__ __forceinline__ void stacked_body(const CUtensorMap* tmA0, const CUte
           const int kb0 = SPLIT ? t / tiles * P->part_kb : 0;  // 64-wide k sub-tiles kb0 .. kb0 + KB - 1
           const int KB = SPLIT ? min(P->part_kb, (j.KB - 1) * 2 + j.klast - kb0) : (j.KB - 1) * 2 + j.klast;
           const int arow = j.tm * BM, brow = j.tn * 128;
-          const int win = window_len(j.s, (int64_t)j.KB * 128, j.cplx);
+          const int win = window_len(j.s, (int64_t)j.KB * kStackedK, j.cplx);
           int pc = 0;
           for (int wstart = 2, wlen = stk_len0(j.s, win); wstart <= j.s + 1;
                wstart += wlen, wlen = min(win, j.s + 2 - wstart)) {
@@ -804,7 +795,7 @@ __device__ __forceinline__ void stacked_body(const CUtensorMap* tmA0, const CUte
           const TileJob j = get_job<128, 2, GROUPED>(SPLIT ? t % tiles : t, tmA0, tmB0, P, G);
           if (j.skip) continue;
           const int KB = SPLIT ? min(P->part_kb, (j.KB - 1) * 2 + j.klast - t / tiles * P->part_kb) : (j.KB - 1) * 2 + j.klast;
-          const int win = window_len(j.s, (int64_t)j.KB * 128, j.cplx);
+          const int win = window_len(j.s, (int64_t)j.KB * kStackedK, j.cplx);
           for (int wstart = 2, wlen = stk_len0(j.s, win); wstart <= j.s + 1;
                wstart += wlen, wlen = min(win, j.s + 2 - wstart)) {
             for (int q = 0; q < (wlen + 1) / 2; ++q) {
@@ -935,7 +926,7 @@ __device__ __forceinline__ void stacked_body(const CUtensorMap* tmA0, const CUte
       const bool row_ok = grow < j.rows;
       const int64_t orow = j.cplx ? (grow >> 1) : grow;
       const int e_row = (row_ok && j.e != nullptr) ? j.e[orow] : 0;
-      const int win = window_len(s, (int64_t)j.KB * 128, j.cplx);
+      const int win = window_len(s, (int64_t)j.KB * kStackedK, j.cplx);
       const int nout = j.cplx ? NOUT / 2 : NOUT;
       PushArgs pa;
       pa.S0 = reinterpret_cast<long long*>(Rbase) + (size_t)(j.cplx ? chalf * NOUT / 2 : chalf * NOUT) * BM + r;
@@ -1156,7 +1147,7 @@ __global__ void __launch_bounds__(BM) split_finish_kernel(const GemmArgs P) {
   const int chunks = (P.cplx ? 64 : 128) / kFin;
   TileJob j = get_job<128, 2, false>((int)(blockIdx.x / chunks), nullptr, nullptr, &P, nullptr);
   const int o = (int)(blockIdx.x % chunks) * kFin, r = threadIdx.x;
-  const int win = window_len(j.s, (int64_t)j.KB * 128, j.cplx);
+  const int win = window_len(j.s, (int64_t)j.KB * kStackedK, j.cplx);
   const int64_t grow = (int64_t)j.tm * BM + r;
   PushArgs pa;
   pa.orow = j.cplx ? (grow >> 1) : grow;
@@ -1362,6 +1353,8 @@ cudaError_t launch_slice_gemm(const CUtensorMap& tmA, const CUtensorMap& tmB, co
   if (a.parts > 1) {
     if (a.variant != kStackedVariant || a.exact || a.Gdbg != nullptr || a.s > stacked_max_slices())
       return cudaErrorInvalidValue;
+    for (int x = a.s_dev != nullptr ? 1 : a.s; x <= a.s; ++x)  // every count the launch may run has its words
+      if (stk_windows(x, a.k, a.cplx) > a.part_windows) return cudaErrorInvalidValue;
     launch_pdl(slice_gemm_split_kernel, a.grid, THREADS, stk::SMEM, st, tmA, tmB, a);
     const int64_t tiles = ((a.rows + BM - 1) / BM) * ((a.cols + 127) / 128);
     launch_pdl(split_finish_kernel, (unsigned)(tiles * ((a.cplx ? 64 : 128) / kFin)), BM, 0, st, a);

@@ -8,6 +8,7 @@
 #include <sstream>
 
 #include "ozg_context.h"
+#include "ozg_window.h"
 
 namespace ozg {
 
@@ -176,7 +177,7 @@ int choose_variant(ozg_ctx* c, int64_t rows, int64_t cols, int64_t k, int s) {
   return heuristic_variant(rows, cols, k, s);
 }
 
-// How one call runs when no variant is forced or tuned: on difference planes (ozg_gemm_kd.cu) or on
+// How one call runs when no variant is forced: on difference planes (ozg_gemm_kd.cu) or on
 // the stacked kernel, there possibly with every tile's k range cut into parts.  The times of all
 // ways are estimated in microseconds from the tiles in whole waves and the costs measured per
 // 64-wide k stage, per pass and per tile.
@@ -192,27 +193,24 @@ int choose_variant(ozg_ctx* c, int64_t rows, int64_t cols, int64_t k, int s) {
 // / 1024: 1.10 / 1.36, 3616^3 1.51.  Parts against whole tiles (whole calls, us): 256^3 s = 7 72 ->
 // 53, 148 x 100 x 4287 s = 10 705 -> 76, 1537 x 2001 x 1111 s = 10 (208 tiles: a second wave of 56)
 // 455 -> 389, 1024^3 s = 8 154 -> 109; 144 complex tiles of 768^3 s = 6 103 -> 123 in two parts: whole.
-SinglePlan plan_single(ozg_ctx* c, bool cplx, int64_t rows, int64_t cols, int64_t k, int s, int s_planes) {
+SinglePlan plan_single(int num_sms, bool cplx, int64_t rows, int64_t cols, int64_t k, int s, int s_planes) {
   SinglePlan P;
-  if (c->force_variant >= 0 || c->exact || s_planes > stacked_max_slices()) return P;
+  if (s_planes > stacked_max_slices()) return P;
   const bool learned = s != s_planes;
   const int64_t KB = (k + 63) / 64;
-  auto window = [&](int x) {  // window_len of ozg_round.cuh
-    const unsigned long long gmax = (unsigned long long)x * (unsigned long long)(KB * 64) * 16129ull * (cplx ? 2 : 1);
-    return std::max((62 - (64 - __builtin_clzll(gmax))) / 7 + 1, 1);
-  };
+  auto window = [&](int x) { return window_len(x, KB * 64, cplx); };  // of the difference-plane kernel
   auto waves = [](int64_t tiles, int64_t units) { return (double)((tiles + units - 1) / units); };
   const int se = learned ? std::min(s, 8) : s;  // a learned count is 7 - 9 in practice
   int stages = 0;  // of the stacked kernel per 64-wide k sub-tile: groups in pairs from the last down
   for (int g = se + 1; g >= 2; g -= 2) stages += g - 1;
   const int64_t tiles = ((rows + 127) / 128) * ((cols + 127) / 128);
-  double best = waves(tiles, c->num_sms) * (0.275 * stages * (double)KB + 18.0);
-  const int nwin = (se + window(se) - 1) / window(se);
+  double best = waves(tiles, num_sms) * (0.275 * stages * (double)KB + 18.0);
+  const int nwin = stk_windows(se, k, cplx);
   int64_t max_parts = std::min<int64_t>(KB, 64);
   for (int64_t p = 2; p <= max_parts; ++p) {
     const int64_t kb = (KB + p - 1) / p;
     if ((KB + kb - 1) / kb != p) continue;  // the same cut as with fewer parts
-    const double t = waves(tiles * p, c->num_sms) * (0.275 * stages * (double)kb + 3.0 * nwin + 6.0) + 8.0 +
+    const double t = waves(tiles * p, num_sms) * (0.275 * stages * (double)kb + 3.0 * nwin + 6.0) + 8.0 +
                      0.1 * (double)(tiles * nwin);
     if (t < best) {
       best = t;
@@ -220,14 +218,14 @@ SinglePlan plan_single(ozg_ctx* c, bool cplx, int64_t rows, int64_t cols, int64_
       P.part_kb = (int)kb;
     }
   }
-  for (int x = 1; x <= s_planes; ++x) P.part_windows = std::max(P.part_windows, (x + window(x) - 1) / window(x));
+  for (int x = 1; x <= s_planes; ++x) P.part_windows = std::max(P.part_windows, stk_windows(x, k, cplx));
   // difference planes: the exact sum must fit two windows, and R its int32
   auto fits = [&](int x) { return x <= 2 * window(x) && window(x) * k * (cplx ? 2 : 1) <= 130000; };
   int kd = std::min(s, kKdMax);
   while (kd > 0 && !fits(kd)) --kd;
   if (kd < (learned ? se : s) || kd == 0) return P;  // a fixed count runs on one kernel
   const int products = se + se * se / 4, win = window(se), len0 = se <= win ? 0 : se - win;
-  const double diff = waves(kd_tiles(rows, cols), c->num_sms / 2) *
+  const double diff = waves(kd_tiles(rows, cols), num_sms / 2) *
                           (0.30 * products * (double)KB + (cplx ? 2 * se - 1 + 25.0 : 3.3 * (2 * se - 1 + len0) + 36.0)) +
                       (double)(rows + cols) * (double)k * 2.0 * (products - se) / 5.5e6;
   if (diff < best) P.kd = kd;

@@ -10,6 +10,8 @@
 #pragma once
 #include <cstdint>
 
+#include "ozg_window.h"
+
 namespace ozg {
 
 // RN(|N| 2^E) with the sign applied, for |N| = (mh, ml) != 0, |N| < 2^127.  The ulp of the
@@ -68,21 +70,7 @@ __device__ __forceinline__ double round_i128(int64_t hi, uint64_t lo, int E) {
   return __longlong_as_double(neg ? (rb | (long long)0x8000000000000000ull) : rb);
 }
 
-// ---- integer windows (default epilogue) ----------------------------------------------------
-// The group sums enter R by Horner's rule in exact int64 arithmetic, c consecutive groups per
-// window, where c is the largest count whose worst case stays below 2^63:
-//   |G_g| <= (g - 1) * kpad * 127^2 (x2 for the complex combine) <= gmax < 2^L,
-//   |window| <= gmax (128^c - 1) / 127 < 2^(L + 7 c) / 127 <= 2^69 / 127   with
-//   c = (62 - L) / 7 + 1, i.e. L + 7 c <= 69: below 2^62 (128/127) < 2^63 - 2^57.
-// Two windows form the exact 128-bit N = W0 128^len1 + W1, rounded to FP64 once with integer
-// instructions only; a third and later window continue in FP64 (one rounding per window).
-__device__ __forceinline__ int window_len(int s, int64_t kpad, int cplx) {
-  const unsigned long long gmax = (unsigned long long)s * (unsigned long long)kpad * 16129ull * (cplx ? 2ull : 1ull);
-  const int L = 64 - __clzll((long long)gmax);
-  const int c = (62 - L) / 7 + 1;
-  return c < 1 ? 1 : c;
-}
-
+// ---- integer windows (default epilogue; their lengths: ozg_window.h) -------------------------
 // (a 2^sh + b) as a 128-bit two's complement integer (hi, lo), 1 <= sh <= 63.
 __device__ __forceinline__ void i128_shl_add(long long a, int sh, long long b, long long& hi, unsigned long long& lo) {
   lo = (unsigned long long)a << sh;

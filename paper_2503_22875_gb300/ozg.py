@@ -87,6 +87,7 @@ def load():
     L.ozg_dgemm_grouped_host.argtypes = [vp, i64, vp, vp, vp]
     L.ozg_set_host_parts.argtypes = [vp, i32]
     L.ozg_zgemm3m.argtypes = [vp, ch, ch, i64, i64, i64, vp, vp, i64, vp, i64, vp, vp, i64, i32, vp]
+    L.ozg_debug_single_plan.argtypes = [i32, i32, i64, i64, i64, i32, i32, i32, vp]
     L.ozg_debug_wait.argtypes = [vp, ctypes.c_longlong]
     L.ozg_debug_fail_allocs.argtypes = [vp, i32]
     L.ozg_dgemm_regions.argtypes = [vp, ch, ch, i64, i64, i64, dbl, vp, i64, vp, i64, dbl, vp, i64, i32, i32, vp]
@@ -113,6 +114,14 @@ def kernel_launches() -> int:
     n = ctypes.c_longlong(0)
     _check(load().ozg_kernel_launches(ctypes.byref(n)), "ozg_kernel_launches")
     return int(n.value)
+
+
+def single_plan(num_sms, complex_, m, n, k, slices, sel_max=0, fallback=0) -> dict:
+    """How a single call is planned on a device of num_sms SMs (ozg_debug_single_plan; no GPU needed)."""
+    p = (ctypes.c_int * 4)()
+    _check(load().ozg_debug_single_plan(int(num_sms), int(bool(complex_)), m, n, k, int(slices), int(sel_max),
+                                        int(fallback), p), "ozg_debug_single_plan")
+    return dict(zip(("kd", "parts", "part_kb", "part_windows"), p))
 
 
 def strerror(code: int) -> str:
