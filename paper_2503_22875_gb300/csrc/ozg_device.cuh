@@ -55,6 +55,14 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
   }
 }
 
+// The same for a converged warp whose lanes wait together while one of them issues: no lane goes on
+// before all have seen the phase.  Each lane polls by itself and the loop need not reconverge, so
+// without the vote the issuing lane could run ahead of one still polling; after a trip round the ring
+// the barrier's parity is again the one that lane waits for, and it would wait until the time-out.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int* status) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, status));
+}
+
 // ------------------------------------------------------------------------------ TMA
 __device__ __forceinline__ void tma_load_3d(const CUtensorMap* map, uint64_t* bar, void* smem_dst, int c0, int c1,
                                             int c2) {

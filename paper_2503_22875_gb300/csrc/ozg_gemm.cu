@@ -770,6 +770,9 @@ __device__ __forceinline__ void stacked_body(const CUtensorMap* tmA0, const CUte
       // keep one lane.
       if (!GROUPED || lane == 0) {
         const bool lead = GROUPED || elect_one();
+        auto wait = [&](uint64_t* bar, uint32_t parity, volatile int* ab, int* stat) {
+          return GROUPED ? mbar_wait(bar, parity, ab, stat) : mbar_wait_warp(bar, parity, ab, stat);
+        };
         uint32_t e = 0, eph = 0;
         int eprev = -1;  // ring entry of the previous stage (freed by the next commit)
         const uint32_t dA0 = (uint32_t)umma_desc_sw128(smem + A_OFF), dB0 = (uint32_t)umma_desc_sw128(smem + B_OFF);
@@ -807,7 +810,7 @@ __device__ __forceinline__ void stacked_body(const CUtensorMap* tmA0, const CUte
               int left = 0;        // k sweeps left in the current chain
               for (int kbi = 0; kbi < KB; ++kbi) {
                 if (left == 0) {
-                  if (!mbar_wait(&bar_acce[buf], ((acc_par >> buf) & 1) ^ 1, abort_p, status)) goto mma_done;
+                  if (!wait(&bar_acce[buf], ((acc_par >> buf) & 1) ^ 1, abort_p, status)) goto mma_done;
                   tc_fence_after();
                   fresh = true;
                   left = spc;
@@ -817,7 +820,7 @@ __device__ __forceinline__ void stacked_body(const CUtensorMap* tmA0, const CUte
                 if (!two) {
                   // lone group: A_i B_{ga-i} into columns 128 .. 255
                   for (int i = 1; i < ga; ++i) {
-                    if (!mbar_wait(&bar_full[e], eph, abort_p, status)) goto mma_done;
+                    if (!wait(&bar_full[e], eph, abort_p, status)) goto mma_done;
                     tc_fence_after();
                     if (lead) {
                       stk_mma4(dt + 128, dA0 + e * DSLOT, dB0 + e * DSLOT, IDESC1, fresh);
@@ -833,7 +836,7 @@ __device__ __forceinline__ void stacked_body(const CUtensorMap* tmA0, const CUte
                 } else {
                   if (kbi == 0) {
                     // the pass's stage 0: B_ga only, no MMA; it frees the previous stage's entry
-                    if (!mbar_wait(&bar_full[e], eph, abort_p, status)) goto mma_done;
+                    if (!wait(&bar_full[e], eph, abort_p, status)) goto mma_done;
                     tc_fence_after();
                     if (lead && eprev >= 0) umma_commit(&bar_empty[eprev]);
                     eprev = (int)e;
@@ -843,7 +846,7 @@ __device__ __forceinline__ void stacked_body(const CUtensorMap* tmA0, const CUte
                     }
                   }
                   for (int i = 1; i < ga; ++i) {
-                    if (!mbar_wait(&bar_full[e], eph, abort_p, status)) goto mma_done;
+                    if (!wait(&bar_full[e], eph, abort_p, status)) goto mma_done;
                     tc_fence_after();
                     // [B_{ga+1-i}; B_{ga-i}] are adjacent slots (at the ring's end, the last slot
                     // and entry 0's mirror): one N = 256 operand
@@ -860,7 +863,7 @@ __device__ __forceinline__ void stacked_body(const CUtensorMap* tmA0, const CUte
                   }
                   // stage ga: A_ga B_1 (group ga + 1 only) into columns 0 .. 127; its B slot holds
                   // the next sweep's B_ga
-                  if (!mbar_wait(&bar_full[e], eph, abort_p, status)) goto mma_done;
+                  if (!wait(&bar_full[e], eph, abort_p, status)) goto mma_done;
                   tc_fence_after();
                   if (lead) {
                     stk_mma4(dt, dA0 + e * DSLOT, dB0 + (uint32_t)eprev * DSLOT, IDESC1, false);

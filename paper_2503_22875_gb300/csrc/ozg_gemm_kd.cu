@@ -314,7 +314,7 @@ __device__ __forceinline__ void kd_body(const CUtensorMap* tmA0, const CUtensorM
         for (;;) {
           int t;
           if (GROUPED) {
-            if (!mbar_wait(&bar_tfull[tslot], tphase, abort_p, status)) goto mma_done;
+            if (!mbar_wait_warp(&bar_tfull[tslot], tphase, abort_p, status)) goto mma_done;
             t = tile_ring[tslot];
             __syncwarp();
             if (lead) mbar_arrive(&bar_tempty[tslot]);
@@ -336,10 +336,10 @@ __device__ __forceinline__ void kd_body(const CUtensorMap* tmA0, const CUtensorM
             for (; nch > 0; --nch) {
               const int c = (left + nch - 1) / nch;
               left -= c;
-              if (!mbar_wait(&bar_acce[buf], ((acc_par >> buf) & 1) ^ 1, abort_p, status)) goto mma_done;
+              if (!mbar_wait_warp(&bar_acce[buf], ((acc_par >> buf) & 1) ^ 1, abort_p, status)) goto mma_done;
               const uint32_t dt = tmem + (uint32_t)(buf * TN);
               for (int i = 0; i < c; ++i) {
-                if (!mbar_wait(&bar_full[e], eph, abort_p, status)) goto mma_done;
+                if (!mbar_wait_warp(&bar_full[e], eph, abort_p, status)) goto mma_done;
                 tc_fence_after();
                 if (lead) {
                   kd_mma4(dt, dA0 + e * DSLOT, dB0 + e * DSLOT, i != 0);
