@@ -63,7 +63,7 @@ int emu_gemm(ozg_ctx* c, bool cplx, char ta, char tb, int64_t m, int64_t n, int6
   int variant = choose_variant(c, prA, prB, k, s);
   SinglePlan plan;
   if (!Gdbg && c->force_variant < 0 && !c->exact)
-    plan = plan_single(c->num_sms, cplx, prA, prB, k, autos ? std::min(c->sel_s_hi, ozg::kKdMax) : s, s);
+    plan = plan_single(c->num_sms, cplx, prA, prB, k, autos, autos ? std::min(c->sel_s_hi, ozg::kKdMax) : s, s);
   if (!plan.kd && variant != ozg::kStackedVariant) plan.parts = 1;
   const int64_t tiles128 = ((prA + 127) / 128) * ((prB + 127) / 128);
   int kd, nplanes;

@@ -135,15 +135,15 @@ T* gat(ozg_ctx* c, size_t off) {
 // tile variant for one GEMM shape (bit 0: BN = 128, bit 1: deferred pushes): the autotuned
 // choice if known, else the heuristic (least padding; deferral for k >= 2048)
 int choose_variant(ozg_ctx* c, int64_t rows, int64_t cols, int64_t k, int s);
-// how one emulated call without a forced variant or the exact epilogue runs; s: the fixed count or the
-// largest learned one, s_planes: digit planes
+// how one emulated call without a forced variant or the exact epilogue runs; s: the fixed count, or (learned)
+// the largest that can be chosen, s_planes: digit planes
 struct SinglePlan {
   int kd = 0;            // > 0: on difference planes for counts up to kd
   int parts = 1;         // stacked kernel: parts of a tile's k range, of part_kb 64-wide sub-tiles
   int part_kb = 0;
   int part_windows = 0;  // window words per output: those of any count up to s_planes
 };
-SinglePlan plan_single(int num_sms, bool cplx, int64_t rows, int64_t cols, int64_t k, int s, int s_planes);
+SinglePlan plan_single(int num_sms, bool cplx, int64_t rows, int64_t cols, int64_t k, bool learned, int s, int s_planes);
 // grouped calls (ozg_grouped.cu): with sync_reports == false the reports are filled in by
 // grouped_collect_reports once the work has finished
 int grouped_call(ozg_ctx* c, int64_t count, const ozg_gemm_desc* descs, const int* slices, ozg_report* reps,

@@ -52,7 +52,7 @@ extern "C" int ozg_debug_single_plan(int num_sms, int cplx, int64_t m, int64_t n
   const int64_t w = cplx ? 2 : 1;
   const int planes = autos ? std::max(sel_max, fallback) : slices;
   const ozg::host::SinglePlan P =
-      ozg::host::plan_single(num_sms, cplx != 0, w * m, w * n, k, autos ? std::min(sel_max, ozg::kKdMax) : slices, planes);
+      ozg::host::plan_single(num_sms, cplx != 0, w * m, w * n, k, autos, autos ? std::min(sel_max, ozg::kKdMax) : slices, planes);
   plan[0] = P.kd;
   plan[1] = P.kd ? 1 : P.parts;
   plan[2] = P.part_kb;

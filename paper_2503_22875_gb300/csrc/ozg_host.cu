@@ -193,10 +193,9 @@ int choose_variant(ozg_ctx* c, int64_t rows, int64_t cols, int64_t k, int s) {
 // / 1024: 1.10 / 1.36, 3616^3 1.51.  Parts against whole tiles (whole calls, us): 256^3 s = 7 72 ->
 // 53, 148 x 100 x 4287 s = 10 705 -> 76, 1537 x 2001 x 1111 s = 10 (208 tiles: a second wave of 56)
 // 455 -> 389, 1024^3 s = 8 154 -> 109; 144 complex tiles of 768^3 s = 6 103 -> 123 in two parts: whole.
-SinglePlan plan_single(int num_sms, bool cplx, int64_t rows, int64_t cols, int64_t k, int s, int s_planes) {
+SinglePlan plan_single(int num_sms, bool cplx, int64_t rows, int64_t cols, int64_t k, bool learned, int s, int s_planes) {
   SinglePlan P;
   if (s_planes > stacked_max_slices()) return P;
-  const bool learned = s != s_planes;
   const int64_t KB = (k + 63) / 64;
   auto window = [&](int x) { return window_len(x, KB * 64, cplx); };  // of the difference-plane kernel
   auto waves = [](int64_t tiles, int64_t units) { return (double)((tiles + units - 1) / units); };

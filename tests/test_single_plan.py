@@ -52,3 +52,15 @@ def test_words_at_the_padding_edge(call):
     cplx, m, n, k, s = call
     p = ozg.single_plan(SMS, cplx, m, n, k, s)
     assert p["parts"] > 1 and p["part_windows"] == kernel_windows(s, k, cplx)
+
+
+@pytest.mark.parametrize("call", [(False, 2500, 3100, 1900), (False, 4096, 4096, 4096), (False, 300, 200, 3000),
+                                  (True, 1800, 1700, 1900), (False, 1537, 2001, 1111)])
+def test_learned_plan_does_not_depend_on_a_low_fallback(call):
+    """A learned call is planned by the counts the selector can choose, whether the fallback count adds
+    digit planes above the selector's largest class (13), ends at it (12) or below."""
+    plans = [ozg.single_plan(SMS, *call, 0, sel_max=12, fallback=f) for f in (13, 12, 10, 7)]
+    how = [(p["kd"], p["parts"], p["part_kb"]) for p in plans]
+    assert how == how[:1] * len(how)
+    if call == (False, 2500, 3100, 1900):
+        assert plans[0]["kd"] == 10
