@@ -62,21 +62,6 @@ static_assert(SMEM < (1u << 18), "descriptor start addresses stay within their 1
 __device__ __forceinline__ int kd_chains(int n) { return (n + kd::CHAIN_STAGES - 1) / kd::CHAIN_STAGES; }
 // Groups of the first window: all of them when they fit one, else as few as the second leaves.
 __device__ __forceinline__ int kd_len0(int s, int win) { return s <= win ? s : s - win; }
-// sum_{j=0}^{n} 128^j
-__device__ __forceinline__ unsigned long long kd_geom(int n) {
-  unsigned long long w = 1;
-  for (int i = 0; i < n; ++i) w = (w << 7) + 1;
-  return w;
-}
-
-// w as wh 2^32 + wl with a signed low word: v w = (int64) v wl + (v wh) 2^32 (mod 2^64)
-struct KdWeight {
-  int wl, wh;
-};
-__device__ __forceinline__ KdWeight kd_weight(unsigned long long w) {
-  const int wl = (int)(uint32_t)w;
-  return {wl, (int)((long long)(w - (unsigned long long)(long long)wl) >> 32)};
-}
 
 // The four K = 16 MMAs of one 64-wide k sub-tile; the first overwrites the accumulator when it
 // starts a chain.
@@ -84,12 +69,6 @@ __device__ __forceinline__ void kd_mma4(uint32_t dt, uint32_t da, uint32_t db, b
   umma_f16_pair_lo(dt, da, db, kd::IDESC, accumulate ? 1u : 0u);
 #pragma unroll
   for (int k16 = 1; k16 < BK / 16; ++k16) umma_f16_pair_lo(dt, da + 2 * k16, db + 2 * k16, kd::IDESC, 1u);
-}
-
-// W + v w (mod 2^64)
-__device__ __forceinline__ unsigned long long kd_mac(unsigned long long W, int v, KdWeight w) {
-  W += (unsigned long long)((long long)v * w.wl);
-  return W + ((unsigned long long)(uint32_t)(v * w.wh) << 32);
 }
 
 // One finished chain.  The thread's first NREG outputs keep their window words in registers:

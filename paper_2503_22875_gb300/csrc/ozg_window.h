@@ -1,5 +1,5 @@
-// The epilogues' integer windows (host and device): how many slice groups one int64 word holds and
-// how many words a call's sum takes.  The kernels and the plans that size their buffers use the same
+// The epilogues' integer windows (host and device): how many slice groups one int64 word holds,
+// how many words a call's sum takes, and how the difference-plane kernel's sums enter one.  The kernels and the plans that size their buffers use the same
 // functions on the same padded k.
 #pragma once
 #include <cstdint>
@@ -53,6 +53,30 @@ OZG_HD int stk_len0(int s, int win) {
 OZG_HD int stk_windows(int s, int64_t k, int cplx) {
   const int win = window_len(s, stk_kpad(k), cplx);
   return 1 + (s - stk_len0(s, win) + win - 1) / win;
+}
+
+// ---- weights of the difference-plane kernel's sums in a window word --------------------------
+// sum_{j=0}^{n} 128^j
+OZG_HD unsigned long long kd_geom(int n) {
+  unsigned long long w = 1;
+  for (int i = 0; i < n; ++i) w = (w << 7) + 1;
+  return w;
+}
+
+// w as wh 2^32 + wl with a signed low word: v w = (int64) v wl + (v wh) 2^32 (mod 2^64)
+struct KdWeight {
+  int wl, wh;
+};
+OZG_HD KdWeight kd_weight(unsigned long long w) {
+  const int wl = (int)(uint32_t)w;
+  return {wl, (int)((long long)(w - (unsigned long long)(long long)wl) >> 32)};
+}
+
+// W + v w (mod 2^64); the high product counts modulo 2^32 and is formed unsigned, since v holds up to
+// 64 chains (2^30) and wh several bits
+OZG_HD unsigned long long kd_mac(unsigned long long W, int v, KdWeight w) {
+  W += (unsigned long long)((long long)v * w.wl);
+  return W + ((unsigned long long)((uint32_t)v * (uint32_t)w.wh) << 32);
 }
 
 }  // namespace ozg
