@@ -49,7 +49,7 @@ int emu_gemm(ozg_ctx* c, bool cplx, char ta, char tb, int64_t m, int64_t n, int6
   if (autos) s = std::max(c->sel_s_hi, s_fb);
   const int nsamp = autos ? std::max(c->check_samples, 64) : c->check_samples;
   const bool beta_zero0 = (beta[0] == 0.0 && (!cplx || beta[1] == 0.0));
-  int64_t Kp = ozg::plane_pitch(k, false);
+  int64_t Kp;
   const int64_t prA = cplx ? 2 * m : m, prB = cplx ? 2 * n : n;
   const int BM = ozg::slice_gemm_tile_m();
   auto grid_of = [&](int variant) {
@@ -61,15 +61,18 @@ int emu_gemm(ozg_ctx* c, bool cplx, char ta, char tb, int64_t m, int64_t n, int6
   // difference planes up to kd slices (0: none): a fixed count's own, or every learned count that
   // the difference-plane kernel takes
   int variant = choose_variant(c, prA, prB, k, s);
-  SinglePlan plan;
+  SinglePlan planned;
   if (!Gdbg && c->force_variant < 0 && !c->exact)
-    plan = plan_single(c->num_sms, cplx, prA, prB, k, autos, autos ? std::min(c->sel_s_hi, ozg::kKdMax) : s, s);
-  if (!plan.kd && variant != ozg::kStackedVariant) plan.parts = 1;
+    planned = plan_single(c->num_sms, cplx, prA, prB, k, autos, autos ? std::min(c->sel_s_hi, ozg::kKdMax) : s, s);
+  if (!planned.kd && variant != ozg::kStackedVariant) planned.parts = 1;
   const int64_t tiles128 = ((prA + 127) / 128) * ((prB + 127) / 128);
+  SinglePlan plan;
   int kd, nplanes;
   Carve cv;
   size_t oDA, oDB, oE, oF, oNf, oMA, oMB, oSplit, zero_end, oR, oCold, oHist, oSd, oErr2, oSaved;
-  auto layout = [&]() {
+  auto layout = [&](const SinglePlan& how, bool tight) {
+    plan = how;
+    Kp = ozg::plane_pitch(k, tight);
     kd = plan.kd;
     nplanes = ozg::kd_planes(s, kd);
     const int grid = std::max({grid_of(0), grid_of(1), kd ? grid_kd : 0});  // R scratch for every kernel
@@ -86,15 +89,12 @@ int emu_gemm(ozg_ctx* c, bool cplx, char ta, char tb, int64_t m, int64_t n, int6
     oHist = cv.take(2 * 10 * 8), oSd = cv.take(4 * sizeof(int)), oErr2 = cv.take(sizeof(double));
     oSaved = cv.take((autos && !beta_zero0) ? (size_t)m * n * (cplx ? 16 : 8) : 8);
   };
-  layout();
-  if ((kd || plan.parts > 1) && !ws_available(c, cv.off)) {  // without either where the memory is not there
-    plan = SinglePlan();
-    layout();
-  }
-  if (!ws_available(c, cv.off)) {  // nor for planes on whole 128-byte lines
-    Kp = ozg::plane_pitch(k, true);
-    layout();
-  }
+  // as planned, else digit planes alone on whole 128-byte lines, else on 16-byte rows: what the memory allows
+  layout(SinglePlan(), true);
+  const size_t lean = cv.off;
+  layout(planned, false);
+  if ((kd || plan.parts > 1) && !ws_room(c, lean, cv.off)) layout(SinglePlan(), false);
+  if (!ws_room(c, lean, cv.off)) layout(SinglePlan(), true);
   int rc = ensure_ws(c, cv.off);
   if (rc) return rc;
   cudaStream_t st = c->stream;

@@ -106,10 +106,10 @@ struct Carve {
 };
 
 int ensure_ws(ozg_ctx* c, size_t bytes);
-// whether ensure_ws / ensure_gws would find the memory: the workspace is large enough, or enough is free (and
-// the stream is not being captured, where it cannot grow)
-bool ws_available(ozg_ctx* c, size_t bytes);
-bool gws_available(ozg_ctx* c, size_t bytes);
+// whether the (grouped) workspace may hold a layout of `bytes` for a call that needs `lean`: it does already,
+// or layout_room allows the growth (and the stream is not being captured, where it cannot grow)
+bool ws_room(ozg_ctx* c, size_t lean, size_t bytes);
+bool gws_room(ozg_ctx* c, size_t lean, size_t bytes);
 int ensure_gws(ozg_ctx* c, size_t bytes);  // grouped workspace; bumps gws_epoch when it moves
 int ensure_z3ws(ozg_ctx* c, size_t bytes);  // 3M operands and products
 cudaEvent_t pool_get(ozg_ctx* c);

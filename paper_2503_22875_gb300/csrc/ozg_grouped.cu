@@ -225,8 +225,10 @@ int build_plan(ozg_ctx* c, int64_t count, const ozg_gemm_desc* d, const std::vec
   }
   P->oMax = max0;
   P->max_bytes = cv.off - max0;
+  size_t lines = 0;  // what whole-line rows add
   for (int64_t i = 0; i < count; ++i) {
     const int64_t Kp = plane_pitch(d[i].k, tight);
+    lines += (size_t)planes[i] * (d[i].m + d[i].n) * (Kp - plane_pitch(d[i].k, true)) * 2;
     oEA[i] = cv.take(4 * (size_t)d[i].m);
     oEB[i] = cv.take(4 * (size_t)d[i].n);
     oDA[i] = cv.take((size_t)planes[i] * d[i].m * Kp * 2);
@@ -300,7 +302,7 @@ int build_plan(ozg_ctx* c, int64_t count, const ozg_gemm_desc* d, const std::vec
     }
     P->save_units = sp[count];
   }
-  if (!tight && !gws_available(c, cv.off)) return build_plan(c, count, d, s, TA, TB, autom, variant, P, true);
+  if (lines > 0 && !gws_room(c, cv.off - lines, cv.off)) return build_plan(c, count, d, s, TA, TB, autom, variant, P, true);
   int rc = ensure_gws(c, cv.off);
   if (rc) return rc;
   P->epoch = c->gws_epoch;

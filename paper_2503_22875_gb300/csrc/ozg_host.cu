@@ -47,7 +47,7 @@ static int grow_buffer(ozg_ctx* c, void** buf, size_t* cap, size_t bytes) {
     *buf = nullptr;
     *cap = 0;
   }
-  size_t want = align_up(bytes + bytes / 8, 1 << 20);
+  size_t want = workspace_size(bytes);
   if (c->fail_allocs > 0) {  // injected failure (test hook), as if cudaMalloc had failed
     --c->fail_allocs;
     return OZG_ERR_ALLOC;
@@ -62,7 +62,7 @@ static int grow_buffer(ozg_ctx* c, void** buf, size_t* cap, size_t bytes) {
   return OZG_OK;
 }
 
-static bool room_for(ozg_ctx* c, size_t cap, size_t bytes) {
+static bool room_for(ozg_ctx* c, size_t cap, size_t lean, size_t bytes) {
   if (bytes <= cap) return true;
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(c->stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
@@ -74,11 +74,11 @@ static bool room_for(ozg_ctx* c, size_t cap, size_t bytes) {
     cudaGetLastError();
     return false;
   }
-  return bytes + bytes / 8 + ((size_t)64 << 20) <= free_b + cap;
+  return layout_room(cap, lean, bytes, free_b);
 }
 
-bool ws_available(ozg_ctx* c, size_t bytes) { return room_for(c, c->ws_cap, bytes); }
-bool gws_available(ozg_ctx* c, size_t bytes) { return room_for(c, c->gws_cap, bytes); }
+bool ws_room(ozg_ctx* c, size_t lean, size_t bytes) { return room_for(c, c->ws_cap, lean, bytes); }
+bool gws_room(ozg_ctx* c, size_t lean, size_t bytes) { return room_for(c, c->gws_cap, lean, bytes); }
 
 int ensure_ws(ozg_ctx* c, size_t bytes) { return grow_buffer(c, &c->ws, &c->ws_cap, bytes); }
 int ensure_z3ws(ozg_ctx* c, size_t bytes) { return grow_buffer(c, &c->z3ws, &c->z3ws_cap, bytes); }
