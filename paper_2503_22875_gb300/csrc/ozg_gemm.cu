@@ -1104,7 +1104,7 @@ template <int BN_, int SUB_>
 __global__ void __launch_bounds__(THREADS, 1)
     slice_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                       const GemmArgs P) {
-  pdl_entry();
+  pdl_wait();
   if (P.nonfinite != nullptr && *P.nonfinite) return;  // the native FP64 kernel handles this call
   gemm_body<BN_, SUB_, false>(&tmA, &tmB, &P, nullptr);
 }
@@ -1126,7 +1126,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1) slice_ge
 __global__ void __launch_bounds__(THREADS, 1)
     slice_gemm_stacked_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                               const GemmArgs P) {
-  pdl_entry();
+  pdl_wait();
   if (P.nonfinite != nullptr && *P.nonfinite) return;
   if (P.kd != 0 && P.s_dev != nullptr && *P.s_dev <= P.kd) return;  // the difference-plane launch runs
   stacked_body<false>(&tmA, &tmB, &P, nullptr);
@@ -1135,7 +1135,7 @@ __global__ void __launch_bounds__(THREADS, 1)
 __global__ void __launch_bounds__(THREADS, 1)
     slice_gemm_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                             const GemmArgs P) {
-  pdl_entry();
+  pdl_wait();
   if (P.nonfinite != nullptr && *P.nonfinite) return;
   if (P.kd != 0 && P.s_dev != nullptr && *P.s_dev <= P.kd) return;
   stacked_body<false, true>(&tmA, &tmB, &P, nullptr);

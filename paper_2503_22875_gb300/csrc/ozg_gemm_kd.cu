@@ -533,7 +533,7 @@ template <bool CPLX>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
     slice_gemm_kd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                          const GemmArgs P) {
-  pdl_entry();
+  pdl_wait();
   if (P.nonfinite != nullptr && *P.nonfinite) return;
   if (P.s_dev != nullptr && *P.s_dev > P.kd) return;  // no difference planes: the plane-by-plane launch runs
   kd_body<false, CPLX>(&tmA, &tmB, &P, nullptr);

@@ -17,16 +17,22 @@ namespace ozg {
 long long& launch_counter();
 inline void note_launch() { __atomic_fetch_add(&launch_counter(), 1LL, __ATOMIC_RELAXED); }
 
-// The launches of a single call are programmatic dependents: a kernel is launched once every CTA of
-// its predecessor in the stream has started, and waits in pdl_entry, before its first access to
-// memory, until the predecessor has completed and its writes are visible.  Every kernel launched so
-// starts with pdl_entry in every thread, so the wait carries through the sequence (256^3 s = 7: 53.2
-// -> 40.9 us, complex 768^3 s = 6: 112 -> 100).  The batched kernels are launched plainly: they gained
-// nothing as dependents inside a graph, and beside other streams' work (the parts of a batch in host
-// memory) their waiting CTAs held SMs (2.98 -> 3.28 ms).
+// The launches of a single call are programmatic dependents: a kernel may be launched before its
+// predecessor in the stream has completed, and waits, before its first access to memory, until the
+// predecessor has and its writes are visible.  Every kernel launched so starts with pdl_entry or pdl_wait
+// in every thread, so the wait carries through the sequence.  Waiting CTAs hold SMs that other streams'
+// calls could use, so they are let in late: a short kernel lets its dependent start once it runs itself
+// (pdl_entry), and the digits and the slice products, whose dependents are wide or would wait long, only as
+// their last CTAs end (pdl_wait), which still hides the launch.  us per call, plain launches / dependents
+// let in at a kernel's first instruction / now: 256^3 s = 7 41.2 / 29.5 / 28.0, 2048^3 s = 8 424 / 410 / 404,
+// two contexts on two streams 359 / 389 / 356, 1024^3 s = 8 on two streams 70.6 / 80.2 / 69.3.
+// The batched kernels are launched plainly: they gained nothing as dependents inside a graph, and beside
+// other streams' work (the parts of a batch in host memory) their waiting CTAs held SMs (2.98 -> 3.28 ms).
 #ifdef __CUDACC__
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_entry() {
-  asm volatile("griddepcontrol.launch_dependents;\n griddepcontrol.wait;" ::: "memory");
+  pdl_wait();
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 template <typename... P, typename... A>
 void launch_pdl(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, const A&... args) {

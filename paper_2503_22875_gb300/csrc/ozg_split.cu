@@ -280,7 +280,7 @@ __device__ __forceinline__ void digits_strided(const SplitArgs& J, const PlaneRa
 // which carries the registers and shared memory of the larger path).
 template <int CPLX, int KD, int ROWS>
 __global__ void __launch_bounds__(256) digits_kernel(const SplitArgs a, const SplitArgs b, unsigned blocks_a) {
-  pdl_entry();
+  pdl_wait();
   const bool first = blockIdx.x < blocks_a;
   const SplitArgs& J = first ? a : b;
   const PlaneRange pr{J.plane_from, J.plane_to, J.gate, J.kd, J.diff};
