@@ -283,12 +283,15 @@ int ozg_set_fallback_slices(ozg_ctx* ctx, int slices);
  * (rounded log2 of m, n, k and the slice count; variants 0..3 and 5) or a grouped batch (every
  * variant) is seen, keeps the fastest,
  * and appends single-call choices to cache_path (may be NULL) as "bucket variant" lines that
- * later contexts read back.  Tuning runs only for calls with beta == 0 (C is then write-only);
- * other calls use the heuristic: single calls with at most 16 slices outside the exact epilogue
+ * later contexts read back.  Calls that the heuristic would run on difference planes have buckets of
+ * their own (bit 63 set), in which those are timed too, each way with its split of the operands, and saved
+ * as 6; choices saved for the other buckets, made without them, do not apply to such calls.
+ * Tuning runs only for calls with a fixed slice count and beta == 0 (C is then write-only);
+ * other calls use saved choices or the heuristic: single calls with at most 16 slices outside the exact epilogue
  * run on difference planes (A_p B_q + A_q B_p from three products of which two are shared: s + s^2 / 4
  * products instead of s (s + 1) / 2), or on the stacked group pairs (variant 5), there with few
- * tiles cut along k, whichever a cost model expects to be fastest (the tuner and its saved choices
- * apply to calls that the model leaves on the tile variants); otherwise the width that pads least, then for
+ * tiles cut along k (also where variant 5 is the saved choice), whichever a cost model expects to be fastest;
+ * otherwise the width that pads least, then for
  * 128 x 256 tiles deferral when k >= 2048 (for a grouped batch, the mean k weighted by m n s^2)
  * and for 128 x 128 tiles variant 5 in grouped calls whose slice counts allow it, else two k
  * slices per stage (variant 1). */

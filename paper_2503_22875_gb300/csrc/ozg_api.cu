@@ -64,6 +64,13 @@ int emu_gemm(ozg_ctx* c, bool cplx, char ta, char tb, int64_t m, int64_t n, int6
   SinglePlan planned;
   if (!Gdbg && c->force_variant < 0 && !c->exact)
     planned = plan_single(c->num_sms, cplx, prA, prB, k, autos, autos ? std::min(c->sel_s_hi, ozg::kKdMax) : s, s);
+  if (planned.kd && !autos) {  // the tuner may have found a tile variant faster
+    const auto it = c->tune.find(shape_bucket(prA, prB, k, s) | kDiffBucket);
+    if (it != c->tune.end() && it->second != kDiffChoice) {
+      variant = it->second;
+      planned.kd = 0;
+    }
+  }
   if (!planned.kd && variant != ozg::kStackedVariant) planned.parts = 1;
   const int64_t tiles128 = ((prA + 127) / 128) * ((prB + 127) / 128);
   SinglePlan plan;
@@ -202,37 +209,86 @@ int emu_gemm(ozg_ctx* c, bool cplx, char ta, char tb, int64_t m, int64_t n, int6
   ga.s_dev = autos ? s_dev : nullptr;
   ga.exact = c->exact;
   ga.kd = kd;
-  if (c->autotune && !kd && c->force_variant < 0 && !Gdbg && ga.beta_zero && !autos) {
-    const uint64_t bucket = shape_bucket(prA, prB, k, s);
+  // the call on tile variant v, cut along k where planned
+  auto on_tiles = [&](ozg::GemmArgs g, int v) {
+    g.variant = v;
+    g.defer = ozg::variant_defers(v);
+    g.grid = grid_of(v);
+    if (!plan.kd && plan.parts > 1 && v == ozg::kStackedVariant) {
+      g.parts = plan.parts;
+      g.part_kb = plan.part_kb;
+      g.part_windows = plan.part_windows;
+      g.Wsplit = at<unsigned long long>(c, oSplit);
+      g.grid = (int)std::min<int64_t>(tiles128 * plan.parts, c->num_sms);
+    }
+    return g;
+  };
+  ozg::GemmArgs gd = ga;  // on difference planes
+  gd.grid = grid_kd;
+  if (c->autotune && c->force_variant < 0 && !Gdbg && ga.beta_zero && !autos) {
+    const uint64_t bucket = shape_bucket(prA, prB, k, s) | (kd ? kDiffBucket : 0);
     if (c->tune.find(bucket) == c->tune.end()) {
       // time the 1-CTA variants (two widths x stage shape or deferred pushes, and the stacked
-      // group pairs) on this call (C is write-only here and every variant gives the same bits)
-      float best = 1e30f;
+      // group pairs) on this call (C is write-only here and every variant gives the same bits); where
+      // difference planes are planned also those, either way with the digits pass that writes its planes
+      auto timed = [&](auto&& launch, float& ms) {
+        cudaEvent_t e0 = pool_get(c), e1 = pool_get(c);
+        cudaError_t e = e0 && e1 ? cudaEventRecord(e0, st) : cudaErrorMemoryAllocation;
+        if (e == cudaSuccess) e = launch();
+        if (e == cudaSuccess) e = cudaEventRecord(e1, st);
+        if (e == cudaSuccess) e = cudaEventSynchronize(e1);
+        if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
+        if (e0) c->pool.push_back(e0);
+        if (e1) c->pool.push_back(e1);
+        return e;
+      };
+      float best = 1e30f, split = 0.f, ms = 0.f;
+      int choice = variant;
+      ozg::SplitArgs pa = sa, pb = sb;  // the digit planes alone
+      CUtensorMap pmA = tmA, pmB[2] = {tmB[0], tmB[1]};
+      if (kd) {
+        OZG_CUDA(timed([&] { return ozg::launch_digits_pair(sa, sb, st); }, split));
+        OZG_CUDA(timed([&] { return ozg::launch_slice_gemm_kd(tmA, tmB[1], gd, st); }, ms));
+        best = split + ms;
+        choice = kDiffChoice;
+        pa.kd = pb.kd = pa.diff = pb.diff = 0;
+        OZG_CUDA(timed([&] { return ozg::launch_digits_pair(pa, pb, st); }, split));
+        OZG_CUDA(ozg::make_digit_tmap(&pmA, pa.D, k, prA, Kp, s, BM));
+        for (int w : {0, 1}) OZG_CUDA(ozg::make_digit_tmap(&pmB[w], pb.D, k, prB, Kp, s, ozg::slice_gemm_tile_n_of(w)));
+      }
       for (int v : {0, 1, 2, 3, ozg::kStackedVariant}) {
         if (v == ozg::kStackedVariant && (s > ozg::stacked_max_slices() || c->exact)) continue;
-        ozg::GemmArgs gt = ga;
-        gt.variant = v;
-        gt.defer = ozg::variant_defers(v);
-        gt.grid = grid_of(v);
-        cudaEvent_t e0 = pool_get(c), e1 = pool_get(c);
-        if (!e0 || !e1) return OZG_ERR_CUDA;
-        OZG_CUDA(cudaEventRecord(e0, st));
-        cudaError_t le = ozg::launch_slice_gemm(tmA, tmB[v & 1], gt, st);
-        OZG_CUDA(cudaEventRecord(e1, st));
-        float ms = 1e30f;
-        if (le == cudaSuccess && cudaEventSynchronize(e1) == cudaSuccess) cudaEventElapsedTime(&ms, e0, e1);
-        c->pool.push_back(e0);
-        c->pool.push_back(e1);
-        OZG_CUDA(le);
-        if (ms < best) {
-          best = ms;
-          variant = v;
+        ozg::GemmArgs gt = on_tiles(ga, v);
+        gt.kd = 0;
+        auto zero_words = [&] {  // a cut call adds to its words
+          return gt.parts > 1 ? cudaMemsetAsync(gt.Wsplit, 0, zero_end - oSplit, st) : cudaSuccess;
+        };
+        OZG_CUDA(timed(
+            [&] {
+              const cudaError_t e = zero_words();
+              return e == cudaSuccess ? ozg::launch_slice_gemm(pmA, pmB[v & 1], gt, st) : e;
+            },
+            ms));
+        OZG_CUDA(zero_words());
+        if (split + ms < best) {
+          best = split + ms;
+          choice = v;
         }
       }
-      tune_store(c, bucket, variant);
-      ga.variant = variant;
-      ga.defer = ozg::variant_defers(variant);
-      ga.grid = grid_of(variant);
+      tune_store(c, bucket, choice);
+      if (choice == kDiffChoice) {
+        OZG_CUDA(ozg::launch_digits_pair(sa, sb, st));
+      } else {
+        variant = choice;
+        kd = 0;
+        tmA = pmA;
+        tmB[0] = pmB[0];
+        tmB[1] = pmB[1];
+        ga.kd = 0;
+        ga.variant = variant;
+        ga.defer = ozg::variant_defers(variant);
+        ga.grid = grid_of(variant);
+      }
     }
   }
   ozg::CheckArgs ck;
@@ -272,23 +328,9 @@ int emu_gemm(ozg_ctx* c, bool cplx, char ta, char tb, int64_t m, int64_t n, int6
   }
   {
     PhaseScope ps(c, OZG_PHASE_GEMM);
-    if (kd) {
-      ozg::GemmArgs gd = ga;
-      gd.grid = grid_kd;
-      OZG_CUDA(ozg::launch_slice_gemm_kd(tmA, tmB[1], gd, st));  // tmB[1]: boxes of 128 columns
-    }
+    if (kd) OZG_CUDA(ozg::launch_slice_gemm_kd(tmA, tmB[1], gd, st));  // tmB[1]: boxes of 128 columns
     // a learned count above kd runs on the digit planes alone
-    if (!kd || (autos && s > kd)) {
-      ozg::GemmArgs gp = ga;
-      if (!kd && plan.parts > 1 && ga.variant == ozg::kStackedVariant) {
-        gp.parts = plan.parts;
-        gp.part_kb = plan.part_kb;
-        gp.part_windows = plan.part_windows;
-        gp.Wsplit = at<unsigned long long>(c, oSplit);
-        gp.grid = (int)std::min<int64_t>(tiles128 * plan.parts, c->num_sms);
-      }
-      OZG_CUDA(ozg::launch_slice_gemm(tmA, tmB[gp.variant & 1], gp, st));
-    }
+    if (!kd || (autos && s > kd)) OZG_CUDA(ozg::launch_slice_gemm(tmA, tmB[variant & 1], on_tiles(ga, variant), st));
   }
   if (Gdbg) return OZG_OK;
 

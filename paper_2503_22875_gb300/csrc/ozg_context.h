@@ -151,6 +151,10 @@ int grouped_call(ozg_ctx* c, int64_t count, const ozg_gemm_desc* descs, const in
 int grouped_collect_reports(ozg_ctx* c);
 uint64_t shape_bucket(int64_t rows, int64_t cols, int64_t k, int s);
 void tune_store(ozg_ctx* c, uint64_t bucket, int variant);
+// Calls planned on difference planes have a bucket of their own, whose choice is a tile variant or the
+// difference planes: a choice made among the tile variants alone says nothing about such a call.
+constexpr uint64_t kDiffBucket = 1ull << 63;
+constexpr int kDiffChoice = OZG_NUM_TILE_VARIANTS;
 
 }  // namespace host
 }  // namespace ozg
