@@ -1137,7 +1137,6 @@ __global__ void __launch_bounds__(THREADS, 1)
                             const GemmArgs P) {
   pdl_wait();
   if (P.nonfinite != nullptr && *P.nonfinite) return;
-  if (P.kd != 0 && P.s_dev != nullptr && *P.s_dev <= P.kd) return;
   stacked_body<false, true>(&tmA, &tmB, &P, nullptr);
 }
 // Rounds the window sums of the split kernel and writes C: a block per tile and chunk of kFin
@@ -1146,7 +1145,6 @@ constexpr int kFin = 4;
 __global__ void __launch_bounds__(BM) split_finish_kernel(const GemmArgs P) {
   pdl_entry();
   if (P.nonfinite != nullptr && *P.nonfinite) return;
-  if (P.kd != 0 && P.s_dev != nullptr && *P.s_dev <= P.kd) return;
   const int chunks = (P.cplx ? 64 : 128) / kFin;
   TileJob j = get_job<128, 2, false>((int)(blockIdx.x / chunks), nullptr, nullptr, &P, nullptr);
   const int o = (int)(blockIdx.x % chunks) * kFin, r = threadIdx.x;
@@ -1354,7 +1352,7 @@ cudaError_t prepare_kernels() {
 cudaError_t launch_slice_gemm(const CUtensorMap& tmA, const CUtensorMap& tmB, const GemmArgs& a, cudaStream_t st) {
   if (a.grid <= 0) return cudaSuccess;
   if (a.parts > 1) {
-    if (a.variant != kStackedVariant || a.exact || a.Gdbg != nullptr || a.s > stacked_max_slices())
+    if (a.variant != kStackedVariant || a.kd != 0 || a.exact || a.Gdbg != nullptr || a.s > stacked_max_slices())
       return cudaErrorInvalidValue;
     for (int x = a.s_dev != nullptr ? 1 : a.s; x <= a.s; ++x)  // every count the launch may run has its words
       if (stk_windows(x, a.k, a.cplx) > a.part_windows) return cudaErrorInvalidValue;

@@ -113,7 +113,6 @@ __device__ __forceinline__ TileJob get_job(int t, const CUtensorMap* tmA, const 
     j.KB = (int)((c->k + Cfg<BN_, SUB_>::SK - 1) / Cfg<BN_, SUB_>::SK);
     j.klast = (int)((c->k - (int64_t)(j.KB - 1) * Cfg<BN_, SUB_>::SK + BK - 1) / BK);
     j.s = c->s;
-    j.kd = c->kd;
     j.cplx = c->cplx;
     j.skip = (c->nonfinite != nullptr && *c->nonfinite) ? 1 : 0;
     j.rows = c->rows;

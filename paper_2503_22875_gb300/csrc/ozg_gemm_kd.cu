@@ -143,24 +143,20 @@ __device__ __forceinline__ void kd_push(const int (&Gr)[N], long long* W, KdWeig
     kd_push_all<false>(Gr, W, w, std::make_integer_sequence<int, N>());
 }
 
-template <bool GROUPED, bool CPLX>
-__device__ __forceinline__ void kd_body(const CUtensorMap* tmA0, const CUtensorMap* tmB0, const GemmArgs* P,
-                                        const GroupArgs* G) {
+template <bool CPLX>
+__device__ __forceinline__ void kd_body(const CUtensorMap* tmA, const CUtensorMap* tmB, const GemmArgs* P) {
   using namespace kd;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   __shared__ __align__(8) uint64_t bar_full[NE], bar_empty[NE], bar_accf[2], bar_acce[2], bar_done;
-  __shared__ __align__(8) uint64_t bar_tfull[TRING], bar_tempty[TRING];
-  __shared__ int tile_ring[TRING];
   __shared__ uint32_t tmem_slot;
   __shared__ int abort_flag;
 
-  int* status = GROUPED ? G->status : P->status;
-  double* Rws = GROUPED ? G->Rws : P->Rws;
-  const int ntiles = GROUPED ? G->ntiles : (int)(((P->rows + TM - 1) / TM) * ((P->cols + TN - 1) / TN));
+  int* status = P->status;
+  const int ntiles = (int)(((P->rows + TM - 1) / TM) * ((P->cols + TN - 1) / TN));
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // rank 0 (the leader) claims tiles, owns the stage-full, accumulator-empty and tile-ring-empty
-  // barriers that both CTAs arrive at, and issues the pair MMAs
+  // rank 0 (the leader) owns the stage-full and accumulator-empty barriers that both CTAs arrive at,
+  // and issues the pair MMAs
   const uint32_t rank = cluster_ctarank();
   const bool leader = rank == 0;
   const int nunits = (int)(gridDim.x / 2), unit = (int)(blockIdx.x / 2);
@@ -174,17 +170,12 @@ __device__ __forceinline__ void kd_body(const CUtensorMap* tmA0, const CUtensorM
       mbar_init(&bar_acce[b], 2 * EPI_WARPS);
     }
     mbar_init(&bar_done, 1);
-    for (int i = 0; i < TRING; ++i) {
-      mbar_init(&bar_tfull[i], 1);
-      // the leader's MMA lane and epilogue warps, the peer's producer and epilogue warps
-      mbar_init(&bar_tempty[i], 2 + 2 * EPI_WARPS);
-    }
     abort_flag = 0;
     mbar_fence_init();
   }
-  if (!GROUPED && warp == 0 && lane == 0) {
-    tma_prefetch_desc(tmA0);
-    tma_prefetch_desc(tmB0);
+  if (warp == 0 && lane == 0) {
+    tma_prefetch_desc(tmA);
+    tma_prefetch_desc(tmB);
   }
   if (warp == 1) tmem_alloc_pair(&tmem_slot, 512);
   tc_fence_before();
@@ -202,44 +193,8 @@ __device__ __forceinline__ void kd_body(const CUtensorMap* tmA0, const CUtensorM
       if (lane == 0) {
         uint32_t e = 0, eph = 0;
         long long issued = 0;
-        const CUtensorMap* last_map = nullptr;
-        uint32_t tslot = 0, tphase = 0;
-        int tnext = unit;
-        for (;;) {
-          int t;
-          if (GROUPED && leader) {
-            if (!mbar_wait_cluster(&bar_tempty[tslot], tphase ^ 1, abort_p, status)) goto producer_done;
-            t = tnext < ntiles ? tnext : -1;
-            tile_ring[tslot] = t;
-            mbar_arrive(&bar_tfull[tslot]);
-            st_shared_cluster(mapa_shared(&tile_ring[tslot], 1), t);
-            mbar_arrive_cluster(mapa_shared(&bar_tfull[tslot], 1));  // release: the slot write first
-            if (++tslot == TRING) {
-              tslot = 0;
-              tphase ^= 1;
-            }
-            if (t >= 0) tnext = nunits + atomicAdd(G->tile_counter, 1);
-          } else if (GROUPED) {
-            if (!mbar_wait_cluster(&bar_tfull[tslot], tphase, abort_p, status)) goto producer_done;
-            t = tile_ring[tslot];
-            // the release of the slot depends on the value read, so it cannot overtake the load
-            if (t != INT_MIN) mbar_arrive_remote(mapa_shared(&bar_tempty[tslot], 0));
-            if (++tslot == TRING) {
-              tslot = 0;
-              tphase ^= 1;
-            }
-          } else {
-            t = tnext < ntiles ? tnext : -1;
-            tnext += nunits;
-          }
-          if (t < 0) break;
-          const TileJob j = get_job<256, 1, GROUPED, false, TM>(t, tmA0, tmB0, P, G);
-          if (j.skip) continue;
-          if (GROUPED && j.tmA != last_map) {
-            tensormap_acquire(j.tmA);
-            tensormap_acquire(j.tmB);
-            last_map = j.tmA;
-          }
+        for (int t = unit; t < ntiles; t += nunits) {
+          const TileJob j = get_job<256, 1, false, false, TM>(t, tmA, tmB, P, nullptr);
           // this CTA's 128 rows of A and its half of the B columns
           const int arow = j.tm * TM + (int)rank * BM, brow = j.tn * TN + (int)rank * 128;
           const int nplanes = kd_plane_base(j.s + 1);
@@ -288,26 +243,8 @@ __device__ __forceinline__ void kd_body(const CUtensorMap* tmA0, const CUtensorM
         uint32_t acc_par = 0;  // bit b: parity of the next use of TMEM buffer b
         int buf = 0;
         const uint32_t dA0 = (uint32_t)umma_desc_sw128(smem + A_OFF), dB0 = (uint32_t)umma_desc_sw128(smem + B_OFF);
-        uint32_t tslot = 0, tphase = 0;
-        int tnext = unit;
-        for (;;) {
-          int t;
-          if (GROUPED) {
-            if (!mbar_wait_warp(&bar_tfull[tslot], tphase, abort_p, status)) goto mma_done;
-            t = tile_ring[tslot];
-            __syncwarp();
-            if (lead) mbar_arrive(&bar_tempty[tslot]);
-            if (++tslot == TRING) {
-              tslot = 0;
-              tphase ^= 1;
-            }
-          } else {
-            t = tnext < ntiles ? tnext : -1;
-            tnext += nunits;
-          }
-          if (t < 0) break;
-          const TileJob j = get_job<256, 1, GROUPED, false, TM>(t, tmA0, tmB0, P, G);
-          if (j.skip) continue;
+        for (int t = unit; t < ntiles; t += nunits) {
+          const TileJob j = get_job<256, 1, false, false, TM>(t, tmA, tmB, P, nullptr);
           // passes: D_1, then D_t and M_{t+1} for t = 2 .. s
           for (int pass = 1; pass < 2 * j.s; ++pass) {
             const int np = (pass == 1 || !(pass & 1)) ? 1 : ((pass >> 1) + 1) / 2;
@@ -352,31 +289,12 @@ __device__ __forceinline__ void kd_body(const CUtensorMap* tmA0, const CUtensorM
     uint32_t acc_par = 0;
     int buf = 0;
     // the CTA's scratch: two window words per output
-    long long* scratch = reinterpret_cast<long long*>(Rws + (size_t)blockIdx.x * BM * TN * 2);
+    long long* scratch = reinterpret_cast<long long*>(P->Rws + (size_t)blockIdx.x * BM * TN * 2);
     const bool odd = (lane & 1) != 0;
     const uint32_t tl = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(chalf * NCOL);
     const uint32_t rel[2] = {mapa_shared(&bar_acce[0], 0), mapa_shared(&bar_acce[1], 0)};
-    uint32_t tslot = 0, tphase = 0;
-    int tnext = unit;
-    for (;;) {
-      int t;
-      if (GROUPED) {
-        if (!mbar_wait_cluster(&bar_tfull[tslot], tphase, abort_p, status)) goto epi_done;
-        t = tile_ring[tslot];
-        __syncwarp();
-        // the leader's ring slot; the release depends on the value read (see the producer)
-        if (lane == 0 && t != INT_MIN) mbar_arrive_remote(mapa_shared(&bar_tempty[tslot], 0));
-        if (++tslot == TRING) {
-          tslot = 0;
-          tphase ^= 1;
-        }
-      } else {
-        t = tnext < ntiles ? tnext : -1;
-        tnext += nunits;
-      }
-      if (t < 0) break;
-      TileJob j = get_job<256, 1, GROUPED, false, TM>(t, tmA0, tmB0, P, G);
-      if (j.skip) continue;
+    for (int t = unit; t < ntiles; t += nunits) {
+      TileJob j = get_job<256, 1, false, false, TM>(t, tmA, tmB, P, nullptr);
       j.cplx = CPLX;
       const int s = j.s;
       const int win = window_len(s, (int64_t)j.KB * BK, CPLX);
@@ -536,7 +454,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
   pdl_wait();
   if (P.nonfinite != nullptr && *P.nonfinite) return;
   if (P.s_dev != nullptr && *P.s_dev > P.kd) return;  // no difference planes: the plane-by-plane launch runs
-  kd_body<false, CPLX>(&tmA, &tmB, &P, nullptr);
+  kd_body<CPLX>(&tmA, &tmB, &P);
 }
 
 }  // namespace

@@ -128,7 +128,7 @@ struct GroupCall {
   CUtensorMap tmA, tmB;         // digit planes of this call (64-byte aligned inside the struct)
   CUtensorMap tmBh;             // B planes with half-height boxes (the CTA-pair variant)
   int64_t rows = 0, cols = 0, m = 0, n = 0, k = 0;
-  int s = 0, cplx = 0, beta_zero = 1, kd = 0;  // kd: as GemmArgs::kd
+  int s = 0, cplx = 0, beta_zero = 1, pad = 0;
   const int32_t* e = nullptr;
   const int32_t* f = nullptr;
   double* C = nullptr;
