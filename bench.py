@@ -18,8 +18,8 @@ the grouped slice-product kernel, the CPU oracle on a bounded sample, and an end
 with the whole batch copied host -> device and the results device -> host in every step.
 
 roofline.traffic is the per-launch DRAM bytes of the committed one-pass ncu summary under
-profiles/ when it was taken on the current kernel sources (sha256 of ozg_gemm.cu,
-ozg_device.cuh, ozg_internal.h and ozg_round.cuh), else null; a figure taken on other sources
+profiles/ when it was taken on the current kernel sources (the sha256 over
+KERNEL_SOURCES), else null; a figure taken on other sources
 is reported as roofline.traffic_other_source with the hash it was taken on.
 
   python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ozg|reference]
@@ -124,9 +124,14 @@ def measured_peaks():
     return {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0, "bf16_tflops_sustained": 1700.0}, "fallback"
 
 
+# every source that the slice-product kernels are compiled from
+KERNEL_SOURCES = ("ozg_gemm.cu", "ozg_gemm_kd.cu", "ozg_gemm_dev.cuh", "ozg_device.cuh", "ozg_internal.h", "ozg_planes.h",
+                  "ozg_round.cuh", "ozg_window.h")
+
+
 def source_hash():
     h = hashlib.sha256()
-    for f in ("ozg_gemm.cu", "ozg_device.cuh", "ozg_internal.h", "ozg_round.cuh"):
+    for f in KERNEL_SOURCES:
         with open(os.path.join(ROOT, "paper_2503_22875_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()
