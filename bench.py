@@ -561,6 +561,18 @@ def regions_section(ozg, torch, n, steps, cases=((0.5, 4.0), (0.1, 6.0)), bands=
     return out
 
 
+def single_kernel(ozg, sms, n, s):
+    """(kernel, slice products, tile variant) of an n^3 DGEMM at s slices: difference planes take s + s^2 / 4
+    products, the stacked group pairs (variant 5, whole tiles or cut along k) and above 16 slices the
+    one-group kernel the triangle's s (s + 1) / 2."""
+    plan = ozg.single_plan(sms, False, n, n, n, s)
+    if plan["kd"]:
+        return "slice_gemm_kd_kernel", s + s * s // 4, None
+    if s > 16:
+        return "slice_gemm_kernel", s * (s + 1) // 2, None
+    return "slice_gemm_split_kernel" if plan["parts"] > 1 else "slice_gemm_stacked_kernel", s * (s + 1) // 2, 5
+
+
 def single_section(ozg, torch, size, steps, phis=SINGLE_PHIS, slice_list=tuple(range(3, 11))):
     """Config 2: emulated DGEMM size^3, a = (u - 0.5) exp(phi g), phi in {0.5, 2, 4}, s = 3..10:
     TFLOP/s and sampled double-double error per s, the native FP64 kernel, and the roofline of the
@@ -603,13 +615,9 @@ def single_section(ozg, torch, size, steps, phis=SINGLE_PHIS, slice_list=tuple(r
             ph = ctx.phase_times()
             ctx.set_profiling(False)
             gemm_ms = ph["gemm"][0] / max(ph["gemm"][1], 1)
-            # large single calls of at most 12 slices run on difference planes (s + s^2 / 4 products), others
-            # of at most 16 the stacked group pairs (variant 5: the triangle's products)
-            diff = n >= 4096 and s <= 12
-            kname = "slice_gemm_kd_kernel" if diff else "slice_gemm_stacked_kernel" if s <= 16 else "slice_gemm_kernel"
-            products = s + s * s // 4 if diff else s * (s + 1) // 2
-            roof = tensor_roofline(kname, products * flops, gemm_ms, f"slice_gemm_{n}_s{s}",
-                                   5 if s <= 16 and not diff else None)
+            sms = torch.cuda.get_device_properties(torch.cuda.current_device()).multi_processor_count
+            kname, products, variant = single_kernel(ozg, sms, n, s)
+            roof = tensor_roofline(kname, products * flops, gemm_ms, f"slice_gemm_{n}_s{s}", variant)
             roof["slices"] = s
             roof["algorithmic_bytes"] = 2.0 * s * 2 * n * n + 8.0 * n * n
             ms_nat = timed(torch, st, lambda: ctx.native_dgemm("N", "N", n, n, n, 1.0, dA, n, dB, n, 0.0, dC, n), 1,

@@ -1,0 +1,15 @@
+"""The kernel and product count that bench.py's single-call roofline names are those of the call's plan."""
+import pytest
+
+import bench
+from paper_2503_22875_gb300 import build, ozg
+
+
+@pytest.mark.parametrize("n,s,kernel,products", [
+    (8192, 7, "kd", 19), (4096, 10, "kd", 35), (4096, 11, "stacked", 66), (8192, 12, "stacked", 78),
+    (32768, 7, "stacked", 28), (1024, 8, "split", 36), (4096, 18, "", 171)])
+def test_kernel_of_a_single_call(n, s, kernel, products):
+    build.build()
+    name, count, variant = bench.single_kernel(ozg, 152, n, s)
+    assert (name, count) == (f"slice_gemm_{kernel}_kernel".replace("__", "_"), products)
+    assert variant == (5 if kernel in ("stacked", "split") else None)
