@@ -573,6 +573,12 @@ def single_kernel(ozg, sms, n, s):
     return "slice_gemm_split_kernel" if plan["parts"] > 1 else "slice_gemm_stacked_kernel", s * (s + 1) // 2, 5
 
 
+def single_profile(kernel, n, s):
+    """Name of the committed profile of that kernel on an n^3 DGEMM at s slices."""
+    kind = {"slice_gemm_kd_kernel": "kd_", "slice_gemm_split_kernel": "split_"}.get(kernel, "")
+    return f"slice_gemm_{kind}{n}_s{s}"
+
+
 def single_section(ozg, torch, size, steps, phis=SINGLE_PHIS, slice_list=tuple(range(3, 11))):
     """Config 2: emulated DGEMM size^3, a = (u - 0.5) exp(phi g), phi in {0.5, 2, 4}, s = 3..10:
     TFLOP/s and sampled double-double error per s, the native FP64 kernel, and the roofline of the
@@ -617,7 +623,7 @@ def single_section(ozg, torch, size, steps, phis=SINGLE_PHIS, slice_list=tuple(r
             gemm_ms = ph["gemm"][0] / max(ph["gemm"][1], 1)
             sms = torch.cuda.get_device_properties(torch.cuda.current_device()).multi_processor_count
             kname, products, variant = single_kernel(ozg, sms, n, s)
-            roof = tensor_roofline(kname, products * flops, gemm_ms, f"slice_gemm_{n}_s{s}", variant)
+            roof = tensor_roofline(kname, products * flops, gemm_ms, single_profile(kname, n, s), variant)
             roof["slices"] = s
             roof["algorithmic_bytes"] = 2.0 * s * 2 * n * n + 8.0 * n * n
             ms_nat = timed(torch, st, lambda: ctx.native_dgemm("N", "N", n, n, n, 1.0, dA, n, dB, n, 0.0, dC, n), 1,

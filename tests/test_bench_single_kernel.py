@@ -13,3 +13,10 @@ def test_kernel_of_a_single_call(n, s, kernel, products):
     name, count, variant = bench.single_kernel(ozg, 152, n, s)
     assert (name, count) == (f"slice_gemm_{kernel}_kernel".replace("__", "_"), products)
     assert variant == (5 if kernel in ("stacked", "split") else None)
+
+
+def test_a_profile_is_that_of_the_kernel():
+    kernels = [f"slice_gemm_{x}_kernel" for x in ("kd", "split", "stacked")]
+    names = [bench.single_profile(x, 8192, 7) for x in kernels]
+    assert names == ["slice_gemm_kd_8192_s7", "slice_gemm_split_8192_s7", "slice_gemm_8192_s7"]
+    assert bench.profile_traffic(names[2])[2] == 5  # tile variant 5: the stacked kernel
