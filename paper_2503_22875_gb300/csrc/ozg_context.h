@@ -27,7 +27,7 @@ struct ozg_ctx {
   cudaStream_t stream = nullptr;
   void* ws = nullptr;  // single-call workspace
   size_t ws_cap = 0;
-  int* dflags = nullptr;     // [0] status (sticky until ozg_sync), [1] non-finite flag of the last call
+  int* dflags = nullptr;     // [0] status (sticky until ozg_sync), [1], [2] non-finite flags of the inspection entries
   double* dcheck = nullptr;  // max sampled error of the last call
   int check_samples = 0;
   uint64_t check_seed = 0x5EED;
