@@ -232,9 +232,9 @@ int ozg_set_host_parts(ozg_ctx* ctx, int parts);
  *   P1 = emu(Ar, Br), P2 = emu(Ai, Bi), P3 = emu(Sa, Sb)   (one grouped launch, s slices each)
  *   Re = RN(P1 - P2), Im = RN(RN(P3 - P1) - P2), then alpha and beta as ozg_zgemm.
  * It does 3/4 of the slice products of the triangle; ozg_zgemm, whose calls run on difference planes or cut
- * along k, is the faster form at every size measured (128 to 3616, 5 to 9 slices).  3M has a weaker bound: the error of Im
- * scales with (|Ar| + |Ai|)(|Br| + |Bi|) instead of |Ar||Bi| + |Ai||Br|, and Sa, Sb add one
- * rounding each.  slices: 1..18 or -1 (native FP64, as ozg_zgemm); the learned selector is not
+ * along k, took 0.2 to 1.0 of its time at every size measured (128 to 3616, 5 to 9 slices).  3M has
+ * the weaker error bound: the error of Im scales with (|Ar| + |Ai|)(|Br| + |Bi|) instead of
+ * |Ar||Bi| + |Ai||Br|, and Sa, Sb add one rounding each.  slices: 1..18 or -1 (native FP64, as ozg_zgemm); the learned selector is not
  * used here (0 is invalid, argument 14).  The report's est_err / max_real / max_imag come from
  * the context's sampled check of the complex result.  Workspace: 3 (mk + kn + mn) doubles.
  * Non-finite inputs reach the native kernel per real product. */
@@ -287,7 +287,8 @@ int ozg_set_fallback_slices(ozg_ctx* ctx, int slices);
  * later contexts read back.  Calls that the heuristic would run on difference planes have buckets of
  * their own (bit 63 set), in which those are timed too, each way with its split of the operands, and saved
  * as 6; choices saved for the other buckets, made without them, do not apply to such calls.
- * Tuning runs only for calls with a fixed slice count and beta == 0 (C is then write-only);
+ * Tuning runs only for calls with a fixed slice count and beta == 0 (C is then write-only), and not
+ * while the stream is being captured into a graph;
  * other calls use saved choices or the heuristic: single calls with at most 16 slices outside the exact epilogue
  * run on difference planes (A_p B_q + A_q B_p from three products of which two are shared: s + s^2 / 4
  * products instead of s (s + 1) / 2), or on the stacked group pairs (variant 5), there with few

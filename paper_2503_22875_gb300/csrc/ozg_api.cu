@@ -225,7 +225,7 @@ int emu_gemm(ozg_ctx* c, bool cplx, char ta, char tb, int64_t m, int64_t n, int6
   };
   ozg::GemmArgs gd = ga;  // on difference planes
   gd.grid = grid_kd;
-  if (c->autotune && c->force_variant < 0 && !Gdbg && ga.beta_zero && !autos) {
+  if (c->autotune && c->force_variant < 0 && !Gdbg && ga.beta_zero && !autos && !capturing(c)) {
     const uint64_t bucket = shape_bucket(prA, prB, k, s) | (kd ? kDiffBucket : 0);
     if (c->tune.find(bucket) == c->tune.end()) {
       // time the 1-CTA variants (two widths x stage shape or deferred pushes, and the stacked

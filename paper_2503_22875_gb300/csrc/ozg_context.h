@@ -105,6 +105,7 @@ struct Carve {
   }
 };
 
+bool capturing(ozg_ctx* c);  // whether the context's stream is being captured into a graph
 int ensure_ws(ozg_ctx* c, size_t bytes);
 // whether the (grouped) workspace may hold a layout of `bytes` for a call that needs `lean`: it does already,
 // or layout_room allows the growth (and the stream is not being captured, where it cannot grow)

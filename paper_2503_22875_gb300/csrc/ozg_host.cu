@@ -62,13 +62,16 @@ static int grow_buffer(ozg_ctx* c, void** buf, size_t* cap, size_t bytes) {
   return OZG_OK;
 }
 
+bool capturing(ozg_ctx* c) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(c->stream, &cs) == cudaSuccess) return cs != cudaStreamCaptureStatusNone;
+  cudaGetLastError();
+  return true;
+}
+
 static bool room_for(ozg_ctx* c, size_t cap, size_t lean, size_t bytes) {
   if (bytes <= cap) return true;
-  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(c->stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
-    cudaGetLastError();
-    return false;  // no growing while the caller captures: keep to what was reserved
-  }
+  if (capturing(c)) return false;  // no growing while the caller captures: keep to what was reserved
   size_t free_b = 0, total_b = 0;
   if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
     cudaGetLastError();
@@ -107,8 +110,7 @@ cudaEvent_t pool_get(ozg_ctx* c) {
 PhaseScope::PhaseScope(ozg_ctx* c_, int ph) : c(c_), phase(ph) {
   if (!c->prof) return;
   // no marks inside a graph capture (the replays are timed as a whole)
-  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(c->stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) return;
+  if (capturing(c)) return;
   if ((a = pool_get(c)) != nullptr) cudaEventRecord(a, c->stream);
 }
 

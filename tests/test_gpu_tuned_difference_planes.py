@@ -72,3 +72,34 @@ def test_updates_of_c_are_not_timed(run, tmp_path):
     path = tmp_path / "tune.txt"
     run(path, True, beta=0.5)
     assert not path.exists() or path.read_text() == ""
+
+
+def test_captured_calls_are_not_timed(tmp_path):
+    """A call that is captured into a graph runs as planned: timing it would need the stream."""
+    from paper_2503_22875_gb300 import build, ozg
+    build.build()
+    path = tmp_path / "tune.txt"
+    g = torch.Generator(device="cuda").manual_seed(2)
+    out = []
+    for shape in ((M, N, K, S), (300, 200, 500, 6)):  # difference planes; cut along k
+        m, n, k, s = shape
+        A, B = (torch.rand(x, dtype=torch.float64, device="cuda", generator=g) - 0.5 for x in ((k, m), (n, k)))
+        for capture in (False, True):
+            C = torch.zeros((n, m), dtype=torch.float64, device="cuda")
+            st = torch.cuda.Stream()
+            st.wait_stream(torch.cuda.current_stream())
+            ctx = ozg.Context(1 << 30, stream=st)
+            ctx.set_autotune(capture, str(path))
+            call = lambda: ctx.dgemm("N", "N", m, n, k, 1.0, A, m, B, k, 0.0, C, m, s)
+            if capture:
+                graph = torch.cuda.CUDAGraph()
+                with torch.cuda.graph(graph, stream=st):
+                    call()
+                graph.replay()
+            else:
+                call()
+            torch.cuda.synchronize()
+            ctx.close()
+            out.append(C)
+        assert torch.equal(out[-1], out[-2])
+    assert not path.exists() or path.read_text() == ""
